@@ -135,6 +135,11 @@ def _gauss(points):
     return t(0.5 * (g + 1.0)), t(0.5 * w)
 
 
+def _inv2(J):
+    (a, b), (c, d) = J.tolist()
+    return torch.tensor([[d, -b], [-c, a]], dtype=torch.float64, device=DEV) / (a * d - b * c)
+
+
 def _dg(M, dt):
     """Mass + dt * upwind advection, nodal P2 DG on M x M squares cut in two (as workloads.dg_p2_advection)."""
     h, sq = 1.0 / M, torch.arange(M * M, device=DEV)
@@ -154,7 +159,7 @@ def _dg(M, dt):
            for c in corners]
     for lu in (0, 1):
         c, J = corners[lu], jac[lu]
-        Ji, area = torch.linalg.inv(J), float(torch.linalg.det(J).abs())
+        Ji, area = _inv2(J), h * h
         first = origin + torch.tensor(c[0], dtype=torch.float64, device=DEV) * h
         X = first[:, None, :] + (J @ torch.stack([qx, qy])).T[None]
         bx, by = _flow(X[..., 0], X[..., 1])
@@ -180,7 +185,7 @@ def _dg(M, dt):
             # the edge's points in the neighbour's reference triangle (the mesh is a translate of one square)
             shift = torch.tensor([dx, dy], dtype=torch.float64, device=DEV) * h
             at = t0 + (t1 - t0) * g[:, None] - shift - torch.tensor(corners[k][0], dtype=torch.float64, device=DEV) * h
-            rn = at @ torch.linalg.inv(jac[k]).T
+            rn = at @ _inv2(jac[k]).T
             pn, _ = _p2(rn[:, 0], rn[:, 1])
             blocks[:, lu, e + 1] = dt * torch.einsum("ig,jg,eg->eij", pe, pn, into)
             other[:, lu, e + 1] = torch.where(there, 2 * ((sy + dy) * M + sx + dx) + k, 2 ** 40)
