@@ -1166,17 +1166,27 @@ static void record_cycle(lair_handle *h, Hier &H, int l) {
     if (l == H.bottom_first) {
         const int nl = (int)H.lev.size();
         Level &Z = H.lev[nl - 1];
-        BottomCoarse<T> cz;
-        cz.n = Z.A.nr;
-        cz.Ainv = Z.Ainv;
-        cz.b = B::b(Z);
-        cz.x = B::x(Z, 0);
         const int *seq = relax_seq[h->o.relax];
-        cycle_bottom<T>(static_cast<const BottomLevel<T> *>(H.bottom_desc), nl - 1 - l, cz, seq, h->s);
         int nsw = 0;
         while (nsw < 3 && seq[nsw] >= 0) ++nsw;
         for (int k = l; k < nl - 1; ++k) H.lev[k].xfinal = nsw & 1;
         Z.xfinal = 0;
+        BottomArgs<T> a;
+        a.img = H.bottom_img;
+        a.nl = nl - 1 - l;
+        a.n0 = L.A.nr;
+        a.nc = Z.A.nr;
+        a.o_desc = H.bottom_o.desc;
+        a.o_cb = H.bottom_o.cb;
+        a.o_cx = H.bottom_o.cx;
+        a.o_b0 = H.bottom_o.b0;
+        a.o_x0 = H.bottom_o.x0;
+        a.o_ainv = H.bottom_o.ainv;
+        a.Ainv = Z.Ainv;
+        a.b = B::b(L);
+        a.x = B::x(L, L.xfinal);
+        a.seq = make_int4(seq[0], seq[1], seq[2], 0);
+        cycle_bottom<T>(a, h->s);
         return;
     }
     Level &C = H.lev[l + 1];
@@ -1335,43 +1345,93 @@ static lair_status autotune_views(lair_handle *h, Hier &H) {
 }
 
 // The smallest levels (at most BOTTOM_ROWS rows, below the finest, at least one besides the coarsest) run in the
-// one-CTA bottom kernel: their descriptors in the cycle's precision, uploaded once; the views and buffers they
-// point to live as long as the hierarchy (a refresh refills them in place).
+// one-cluster bottom kernel. Their descriptors are written here in the cycle's precision: the offsets in a CTA's shared
+// memory of the lists, the coarsest inverse and the vectors, whose sizes the host knows; what is left takes view
+// entries (bottom_pack). A bottom whose lists and vectors alone do not fit starts one level further down. The views
+// that the descriptors point to live as long as the hierarchy; a refresh refills them in place and packs the images
+// again.
+template <class T>
+static void pack_bottom(lair_handle *h, Hier &H) {
+    const Level &Z = H.lev.back();
+    bottom_pack<T>(static_cast<const BottomLevel<T> *>(H.bottom_desc), (int)H.lev.size() - 1 - H.bottom_first,
+                   H.bottom_o.desc, H.bottom_o.entries, H.bottom_o.top, Z.A.nr, Z.Ainv, H.bottom_o.ainv, H.bottom_img,
+                   h->s);
+}
+
 template <class T>
 static lair_status prepare_bottom(lair_handle *h, Hier &H) {
-    using B = CycleBufs<T>;
     H.bottom_first = -1;
     const int nl = (int)H.lev.size();
     // (a coarsest level of more than 512 unknowns keeps its many-CTA dense product)
-    if (h->o.nodal > 1 || nl < 3 || H.lev[nl - 1].A.nr > 512) return LAIR_OK;
+    if (h->o.nodal > 1 || nl < 3 || H.lev[nl - 1].A.nr > 512 || !bottom_fits<T>()) return LAIR_OK;
     int first = -1;
     for (int l = 1; l <= nl - 2 && first < 0; ++l)
-        if (H.lev[l].A.nr <= BOTTOM_ROWS) first = l;
+        if (H.lev[l].A.nr <= BOTTOM_ROWS && nl - 1 - l <= BOTTOM_LEVELS) first = l;
     if (first < 0) return LAIR_OK;
-    std::vector<BottomLevel<T>> d(nl - 1 - first);
-    for (int i = 0; i < (int)d.size(); ++i) {
-        Level &L = H.lev[first + i];
-        BottomLevel<T> &t = d[i];
-        t.n = L.A.nr;
-        t.nc = L.nc;
-        t.R = L.Rv;
-        t.P = L.Pv;
-        t.AF = L.AF;
-        t.AC = L.AC;
-        t.p1col = h->o.interp == LAIR_P_ONEPOINT ? L.p1col : nullptr;
-        t.crows = L.crows;
-        t.frows = L.frows;
-        t.b = B::b(L);
-        t.x[0] = B::x(L, 0);
-        t.x[1] = B::x(L, 1);
+    auto &o = H.bottom_o;
+    std::vector<BottomLevel<T>> d;
+    for (; first <= nl - 2; ++first) {
+        d.assign(nl - 1 - first, BottomLevel<T>());
+        int at = 16, top = BOTTOM_SMEM;   // lists from the front, vectors from the back
+        auto take = [&](size_t bytes) {
+            const int p = at;
+            at += (int)((bytes + 15) & ~(size_t)15);
+            return p;
+        };
+        auto take_vec = [&](size_t bytes) { return top -= (int)((bytes + 15) & ~(size_t)15); };
+        auto slices = [](int rows) { return ((rows + 31) / 32 + BOTTOM_CTAS - 1) / BOTTOM_CTAS; };   // of one CTA
+        o.desc = take(sizeof(BottomLevel<T>) * d.size());
+        for (int i = 0; i < (int)d.size(); ++i) {
+            Level &L = H.lev[first + i];
+            BottomLevel<T> &t = d[i];
+            t.n = L.A.nr;
+            t.o_b = take_vec(sizeof(T) * t.n);
+            t.o_x = take_vec(sizeof(T) * t.n);
+            if (h->o.interp == LAIR_P_ONEPOINT) {
+                t.p1col = L.p1col;
+                t.o_p1 = take(sizeof(int16_t) * 32 * slices(t.n));
+            }
+            const SellView *src[4];
+            src[BOTTOM_R] = &L.Rv;
+            src[BOTTOM_P] = &L.Pv;
+            src[BOTTOM_AF] = &L.AF;
+            src[BOTTOM_AC] = &L.AC;
+            for (int k = 0; k < 4; ++k) {
+                const SellView &s = *src[k];
+                BottomView<T> &v = t.v[k];
+                v.nrows = s.nrows;
+                v.ptr = s.slice_ptr;
+                v.row = s.row;
+                v.col = s.col;
+                v.val = static_cast<const T *>(s.val);
+                v.dinv = static_cast<const T *>(s.dinv);
+                if (v.nrows <= 0) continue;
+                v.o_ptr = take(sizeof(int2) * slices(v.nrows));
+                v.o_row = take(sizeof(uint16_t) * 32 * slices(v.nrows));
+                if (v.dinv) v.o_dinv = take(sizeof(T) * 32 * slices(v.nrows));
+            }
+        }
+        const int nz = H.lev[nl - 1].A.nr;
+        o.cb = take_vec(sizeof(T) * nz);
+        o.cx = take_vec(sizeof(T) * nz);
+        const size_t inv = sizeof(double) * (size_t)((nz + BOTTOM_CTAS - 1) / BOTTOM_CTAS) * nz;
+        o.ainv = at + (long long)inv + 64 <= top ? take(inv) : -1;
+        o.entries = (at + 63) & ~63;
+        o.top = top;
+        if (o.entries <= top) break;
     }
+    if (first > nl - 2) return LAIR_OK;
+    o.b0 = d[0].o_b;
+    o.x0 = d[0].o_x;
     const size_t bytes = sizeof(BottomLevel<T>) * d.size();
     char *desc = nullptr;
     TRY(dalloc(h, &desc, bytes));
+    TRY(dalloc(h, &H.bottom_img, (size_t)BOTTOM_SMEM * BOTTOM_CTAS));
     CU(cudaMemcpyAsync(desc, d.data(), bytes, cudaMemcpyHostToDevice, h->s));
-    CU(cudaStreamSynchronize(h->s));
+    // (a copy from pageable memory is staged before cudaMemcpyAsync returns, so d may go)
     H.bottom_desc = desc;
     H.bottom_first = first;
+    pack_bottom<T>(h, H);
     return LAIR_OK;
 }
 
@@ -1680,6 +1740,10 @@ static lair_status refresh_hierarchy(lair_handle *h, Hier &H, const DCsr &Ain) {
             }
         }
         refill_sells(h, H);
+        if (H.bottom_first >= 0) {
+            if (fp32) pack_bottom<float>(h, H);
+            else pack_bottom<double>(h, H);
+        }
         int hc[2];
         TRY(read_ints(h, c2, 2, hc));   // also checks the status word
         H.singular_R = hc[0];

@@ -375,107 +375,327 @@ template void p1_interp<double>(int, const int *, const int *, const uint8_t *, 
                                 cudaStream_t);
 
 // ---------------------------------------------------------------------------------------
-// The bottom of the V-cycle in one CTA: the restrictions of the smallest levels, the coarsest solve, and on the
-// way up their interpolations and F/C sweeps, with a block barrier between phases instead of a kernel boundary.
-// Every row is computed by one thread with the arithmetic of k_sell_spmv, k_sell_sweep, k_p1_interp and
-// k_dense_apply (same entries, same order), so the cycle's result is the same bits either way. Vectors written
-// in one phase and read in a later one are read with plain loads (the block's own writes, ordered by
-// __syncthreads); matrices do not change during the launch. Stopped batched systems are not skipped here.
+// The bottom of the V-cycle in one thread-block cluster: the restrictions of the smallest levels, the coarsest
+// solve, and on the way up their interpolations and F/C sweeps, with a cluster barrier between phases instead of a
+// kernel boundary. Every row is computed by one thread with the arithmetic of k_sell_spmv, k_sell_sweep, k_p1_interp
+// and k_dense_apply (same entries, same order), so the cycle's result is the same bits either way. Stopped batched
+// systems are not skipped here.
+//
+// What bounds it is latency: each phase is a chain slice offset -> column -> gathered x -> fma, which costs 3-8 us a
+// phase as a kernel of its own that reads L2, however few rows there are. So everything the phases read lies in
+// shared memory: slice q of a view belongs to CTA q mod 8, whose part of all levels (row lists, diagonals, entries
+// with 16-bit columns, its rows of the coarsest inverse) lies ready in one contiguous image, packed when the
+// hierarchy is built (k_bottom_pack) and copied with 16-byte cp.async before the kernel waits for its predecessor
+// (the image does not depend on it). Each CTA also holds all vectors of all bottom levels; a row's new value is
+// written into the eight copies through distributed shared memory. Views that do not fit are read from global
+// memory eight entries at a time. Eight CTAs rather than one, because on one SM the FP64 phases and the FP64 coarsest
+// product are bound by its two FP64 lanes (a 128 x 128 product takes 10 us there) and its shared memory ends at
+// about 1,000 rows.
+// Figures: see BOTTOM_ROWS in setup_kernels.cuh.
 // ---------------------------------------------------------------------------------------
 namespace {
 
 template <class T>
-__device__ __forceinline__ void bottom_spmv(const SellView &v, const T *x, T *y) {
-    const T *__restrict__ sval = static_cast<const T *>(v.val);
-    const long long nthr = (long long)((v.nrows + 31) >> 5) * 32;
-    for (long long u = threadIdx.x; u < nthr; u += blockDim.x) {
-        const int lane = (int)(u & 31), sl = (int)(u >> 5), r = sl * 32 + lane;
-        const int a = __ldg(v.slice_ptr + sl);
-        const int base = a + lane, len = (__ldg(v.slice_ptr + sl + 1) - a) >> 5;
-        T acc = T(0);
-        for (int j = 0; j < len; ++j) acc = fma(__ldg(sval + base + 32 * j), x[__ldg(v.col + base + 32 * j)], acc);
-        if (r < v.nrows) y[__ldg(v.row + r)] = acc;
-    }
+__device__ __forceinline__ const T *bottom_at(const unsigned char *sm, int off) {
+    return reinterpret_cast<const T *>(sm + off);
 }
 
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();   // .aligned: the warp arrives as one
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// v at byte offset off of the shared memory of every CTA of the cluster (base[q]: where CTA q's begins)
+__device__ __forceinline__ void bottom_put(const unsigned (&base)[BOTTOM_CTAS], int off, float v) {
+#pragma unroll
+    for (int q = 0; q < BOTTOM_CTAS; ++q)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(base[q] + off), "f"(v) : "memory");
+}
+__device__ __forceinline__ void bottom_put(const unsigned (&base)[BOTTOM_CTAS], int off, double v) {
+#pragma unroll
+    for (int q = 0; q < BOTTOM_CTAS; ++q)
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(base[q] + off), "d"(v) : "memory");
+}
+
+// the sum of this thread's row of the view against x (shared), entries in ascending order as everywhere; warp w of
+// the CTA holds the CTA's w-th slice of the view
 template <class T>
-__device__ __forceinline__ void bottom_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const T *x,
-                                             T *xo) {
-    const T *__restrict__ sval = static_cast<const T *>(v.val);
-    const T *__restrict__ sd = static_cast<const T *>(v.dinv);
-    const long long nthr = (long long)((v.nrows + 31) >> 5) * 32;
-    for (long long u = threadIdx.x; u < nthr + ncopy; u += blockDim.x) {
-        if (u < nthr) {
-            const int lane = (int)(u & 31), sl = (int)(u >> 5), r = sl * 32 + lane;
-            const int a = __ldg(v.slice_ptr + sl);
-            const int base = a + lane, len = (__ldg(v.slice_ptr + sl + 1) - a) >> 5;
-            T acc = T(0);
-            for (int j = 0; j < len; ++j) acc = fma(__ldg(sval + base + 32 * j), x[__ldg(v.col + base + 32 * j)], acc);
-            if (r < v.nrows) {
-                const int i = __ldg(v.row + r);
-                xo[i] = fma(__ldg(sd + r), b[i] - acc, x[i]);
+__device__ __forceinline__ T bottom_row(const unsigned char *sm, const BottomView<T> &v, const T *x) {
+    const int lane = threadIdx.x & 31;
+    const int2 sl = bottom_at<int2>(sm, v.o_ptr)[threadIdx.x >> 5];   // first entry, longest row
+    T acc = T(0);
+    if (v.o_val >= 0) {
+        const uint16_t *col = bottom_at<uint16_t>(sm, v.o_col) + sl.x + lane;
+        const T *val = bottom_at<T>(sm, v.o_val) + sl.x + lane;
+#pragma unroll 4
+        for (int j = 0; j < sl.y; ++j) acc = fma(val[32 * j], x[col[32 * j]], acc);
+    } else {
+        const int *col = v.col + sl.x + lane;
+        const T *val = v.val + sl.x + lane;
+        for (int j = 0; j < sl.y; j += 8) {
+            int c[8];
+            T w[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const bool in = j + k < sl.y;
+                c[k] = in ? __ldg(col + 32 * (j + k)) : 0;
+                w[k] = in ? __ldg(val + 32 * (j + k)) : T(0);
             }
-        } else {
-            const int j = __ldg(copy + (u - nthr));
-            xo[j] = x[j];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (j + k < sl.y) acc = fma(w[k], x[c[k]], acc);
         }
     }
+    return acc;
+}
+
+// y = (view) x, y at byte offset o_y
+template <class T>
+__device__ __forceinline__ void bottom_spmv(const unsigned char *sm, const unsigned (&base)[BOTTOM_CTAS],
+                                            const BottomView<T> &v, const T *x, int o_y) {
+    if ((int)(threadIdx.x >> 5) >= v.nloc) return;
+    const T acc = bottom_row<T>(sm, v, x);
+    const int i = bottom_at<uint16_t>(sm, v.o_row)[threadIdx.x];
+    if (i != BOTTOM_NOROW) bottom_put(base, o_y + i * (int)sizeof(T), acc);
+}
+
+// one Jacobi sweep in place: the new values are written once every CTA has read the old ones
+template <class T>
+__device__ __forceinline__ void bottom_sweep(const unsigned char *sm, const unsigned (&base)[BOTTOM_CTAS],
+                                             const BottomView<T> &v, const T *b, int o_x) {
+    const T *x = bottom_at<T>(sm, o_x);
+    int i = BOTTOM_NOROW;
+    T xn = T(0);
+    if ((int)(threadIdx.x >> 5) < v.nloc) {
+        i = bottom_at<uint16_t>(sm, v.o_row)[threadIdx.x];
+        const T acc = bottom_row<T>(sm, v, x);
+        if (i != BOTTOM_NOROW) xn = fma(bottom_at<T>(sm, v.o_dinv)[threadIdx.x], b[i] - acc, x[i]);
+    }
+    cluster_arrive();
+    cluster_wait();
+    if (i != BOTTOM_NOROW) bottom_put(base, o_x + i * (int)sizeof(T), xn);
+    cluster_arrive();
+    cluster_wait();
 }
 
 }  // namespace
 
+// Lays the image of CTA blockIdx.y out and fills the part of view blockIdx.x (four per level: R, P, AF, AC). The
+// entries of a view go into the image as long as they fit in cap bytes, deepest level first and the F rows (swept
+// twice) before the others; every block works the layout out for itself from the slices' lengths. lv: the levels with
+// the offsets of lists and vectors already set (host). The image starts with its own size, then the descriptors;
+// entries take the bytes from o_entries up to cap. Ainv's rows go to o_ainv (when >= 0).
 template <class T>
-__global__ void __launch_bounds__(BOTTOM_THREADS) k_cycle_bottom(const BottomLevel<T> *__restrict__ lv, int nl,
-                                                                 BottomCoarse<T> cz, int4 seq) {
-    pdl_enter();
-    const int sq[3] = {seq.x, seq.y, seq.z};
-    for (int l = 0; l < nl; ++l) {
-        bottom_spmv<T>(lv[l].R, lv[l].b, l + 1 < nl ? lv[l + 1].b : cz.b);
-        __syncthreads();
+__global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom_pack(const BottomLevel<T> *__restrict__ lv, int nl, int o_desc,
+                                                                int o_entries, int cap, int nz,
+                                                                const double *__restrict__ Ainv, int o_ainv,
+                                                                unsigned char *__restrict__ images) {
+    __shared__ int ofs[4 * BOTTOM_LEVELS], num[4 * BOTTOM_LEVELS], total;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nv = 4 * nl, rank = blockIdx.y;
+    unsigned char *img = images + (size_t)rank * BOTTOM_SMEM;
+    for (int q = w; q < nv; q += BOTTOM_THREADS / 32) {
+        const BottomView<T> &v = lv[q >> 2].v[q & 3];
+        const int s = lane * BOTTOM_CTAS + rank;
+        int c = 32 * s < v.nrows ? v.ptr[s + 1] - v.ptr[s] : 0;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) num[q] = c;
     }
-    {
-        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-        for (int r = threadIdx.x >> 5; r < cz.n; r += nw) {
-            double acc = 0.0;
-            for (int c = lane; c < cz.n; c += 32) acc = fma(__ldg(cz.Ainv + (size_t)r * cz.n + c), (double)cz.b[c], acc);
-            acc = warp_sum(acc);
-            if (lane == 0) cz.x[r] = (T)acc;
-        }
-    }
-    for (int l = nl - 1; l >= 0; --l) {
-        const BottomLevel<T> &L = lv[l];
-        __syncthreads();
-        const T *xc = l + 1 < nl ? lv[l + 1].x[seq.w] : cz.x;
-        if (L.p1col) {
-            for (int i = threadIdx.x; i < L.n; i += blockDim.x) {
-                const int c = __ldg(L.p1col + i);
-                L.x[0][i] = c >= 0 ? xc[c] + T(0) : T(0);
+    __syncthreads();
+    if (t == 0) {
+        const int order[4] = {BOTTOM_AF, BOTTOM_AC, BOTTOM_R, BOTTOM_P};
+        int at = o_entries;
+        for (int l = nl - 1; l >= 0; --l)
+            for (int k = 0; k < 4; ++k) {
+                const int q = 4 * l + order[k];
+                const long long bytes = (long long)num[q] * (int)(sizeof(T) + sizeof(uint16_t));   // a multiple of 64
+                ofs[q] = -1;
+                if (num[q] > 0 && at + bytes <= cap) {
+                    ofs[q] = at;
+                    at += (int)bytes;
+                }
             }
-        } else {
-            bottom_spmv<T>(L.P, xc, L.x[0]);
+        total = at;
+    }
+    __syncthreads();
+    const int q = blockIdx.x;
+    if (q == 0) {
+        if (t < 4) reinterpret_cast<int *>(img)[t] = t == 0 ? total : 0;
+        const int words = nl * (int)(sizeof(BottomLevel<T>) / sizeof(int));
+        for (int k = t; k < words; k += BOTTOM_THREADS)
+            reinterpret_cast<int *>(img + o_desc)[k] = reinterpret_cast<const int *>(lv)[k];
+        __syncthreads();
+        for (int p = t; p < nv; p += BOTTOM_THREADS) {
+            BottomView<T> &v = reinterpret_cast<BottomLevel<T> *>(img + o_desc)[p >> 2].v[p & 3];
+            const int nsl = (v.nrows + 31) >> 5;
+            v.nloc = nsl > rank ? (nsl - rank + BOTTOM_CTAS - 1) / BOTTOM_CTAS : 0;
+            v.o_val = ofs[p];
+            v.o_col = ofs[p] >= 0 ? ofs[p] + num[p] * (int)sizeof(T) : -1;
         }
-        int cur = 0;
-        for (int k = 0; k < 3 && sq[k] >= 0; ++k) {
-            __syncthreads();
-            if (sq[k] == CF_F) bottom_sweep<T>(L.AF, L.crows, L.nc, L.b, L.x[cur], L.x[1 - cur]);
-            else bottom_sweep<T>(L.AC, L.frows, L.n - L.nc, L.b, L.x[cur], L.x[1 - cur]);
-            cur ^= 1;
-        }
+        if (o_ainv >= 0)
+            for (int k = t; k < nz * ((nz - rank + BOTTOM_CTAS - 1) / BOTTOM_CTAS); k += BOTTOM_THREADS)
+                reinterpret_cast<double *>(img + o_ainv)[k] = Ainv[(size_t)(rank + k / nz * BOTTOM_CTAS) * nz + k % nz];
+    }
+    const BottomLevel<T> &L = lv[q >> 2];
+    const BottomView<T> &v = L.v[q & 3];
+    if ((q & 3) == BOTTOM_P && L.p1col) {
+        const int i = (w * BOTTOM_CTAS + rank) * 32 + lane;
+        if (i < L.n) reinterpret_cast<int16_t *>(img + L.o_p1)[t] = (int16_t)L.p1col[i];
+    }
+    // warp w: the CTA's w-th slice
+    const int s = w * BOTTOM_CTAS + rank, u = 32 * s + lane;
+    if (32 * s >= v.nrows) return;
+    reinterpret_cast<uint16_t *>(img + v.o_row)[t] = u < v.nrows ? (uint16_t)v.row[u] : (uint16_t)BOTTOM_NOROW;
+    if (v.dinv && u < v.nrows) reinterpret_cast<T *>(img + v.o_dinv)[t] = v.dinv[u];
+    const int beg = v.ptr[s], len = (v.ptr[s + 1] - beg) >> 5;
+    int loc = 0;   // entries of the CTA's slices before this one
+    for (int k = lane; k < w; k += 32) loc += v.ptr[k * BOTTOM_CTAS + rank + 1] - v.ptr[k * BOTTOM_CTAS + rank];
+    loc = __reduce_add_sync(0xffffffffu, loc);
+    if (lane == 0) reinterpret_cast<int2 *>(img + v.o_ptr)[w] = make_int2(ofs[q] >= 0 ? loc : beg, len);
+    if (ofs[q] < 0) return;
+    T *val = reinterpret_cast<T *>(img + ofs[q]) + loc + lane;
+    uint16_t *col = reinterpret_cast<uint16_t *>(img + ofs[q] + num[q] * (int)sizeof(T)) + loc + lane;
+#pragma unroll 4
+    for (int j = 0; j < len; ++j) {
+        val[32 * j] = v.val[beg + lane + 32 * j];
+        col[32 * j] = (uint16_t)v.col[beg + lane + 32 * j];
     }
 }
 
 template <class T>
-void cycle_bottom(const BottomLevel<T> *lv, int nl, const BottomCoarse<T> &cz, const int *seq3, cudaStream_t s) {
-    int nsw = 0;
-    while (nsw < 3 && seq3[nsw] >= 0) ++nsw;
-    const int4 seq = make_int4(seq3[0], seq3[1], seq3[2], nsw & 1);
-    launch_pdl(k_cycle_bottom<T>, 1, BOTTOM_THREADS, 0, s, lv, nl, cz, seq);
+__global__ void __cluster_dims__(BOTTOM_CTAS, 1, 1) __launch_bounds__(BOTTOM_THREADS) k_cycle_bottom(BottomArgs<T> a) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, rank = blockIdx.x;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const unsigned own = (unsigned)__cvta_generic_to_shared(sm);
+    {
+        const unsigned char *img = a.img + (size_t)rank * BOTTOM_SMEM;
+        const int total = __ldg(reinterpret_cast<const int *>(img));
+        for (int k = 16 * t; k < total; k += 16 * BOTTOM_THREADS)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(own + k), "l"(img + k) : "memory");
+    }
+    unsigned base[BOTTOM_CTAS];
+#pragma unroll
+    for (int q = 0; q < BOTTOM_CTAS; ++q)
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base[q]) : "r"(own), "r"(q));
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int k = t; k < a.n0; k += BOTTOM_THREADS) reinterpret_cast<T *>(sm + a.o_b0)[k] = a.b[k];
+    cluster_arrive();   // every CTA runs and holds its image
+    cluster_wait();
+    const int nl = a.nl;
+    const BottomLevel<T> *lv = bottom_at<BottomLevel<T>>(sm, a.o_desc);
+    for (int l = 0; l < nl; ++l) {
+        bottom_spmv<T>(sm, base, lv[l].v[BOTTOM_R], bottom_at<T>(sm, lv[l].o_b), l + 1 < nl ? lv[l + 1].o_b : a.o_cb);
+        cluster_arrive();
+        cluster_wait();
+    }
+    {
+        // x = Ainv b, row rank + 8 k in this CTA, four rows per warp. A lane sums its columns in ascending order and
+        // the lanes' sums are added in k_dense_apply's butterfly order (16, 8, 4, 2, 1), but four rows share the first
+        // two steps: each half, then each quarter of the warp goes on with its own rows (a warp FP64 instruction
+        // costs 16 cycles of the SM whatever its lanes hold).
+        const int n = a.nc, mine = n > rank ? (n - rank + BOTTOM_CTAS - 1) / BOTTOM_CTAS : 0;
+        const T *cb = bottom_at<T>(sm, a.o_cb);
+        for (int r0 = 4 * w; r0 < mine; r0 += 4 * (BOTTOM_THREADS / 32)) {
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            if (a.o_ainv >= 0) {
+                const double *A = bottom_at<double>(sm, a.o_ainv) + r0 * n;
+#pragma unroll 2
+                for (int c = lane; c < n; c += 32) {
+                    const double xc = (double)cb[c];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (r0 + k < mine) acc[k] = fma(A[k * n + c], xc, acc[k]);
+                }
+            } else {
+                const double *A = a.Ainv + (size_t)(rank + r0 * BOTTOM_CTAS) * n;
+#pragma unroll 4
+                for (int c = lane; c < n; c += 32) {
+                    const double xc = (double)cb[c];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (r0 + k < mine) acc[k] = fma(__ldg(A + (size_t)k * BOTTOM_CTAS * n + c), xc, acc[k]);
+                }
+            }
+            const bool h16 = lane & 16, h8 = lane & 8;
+            const double s0 = __shfl_xor_sync(0xffffffffu, h16 ? acc[0] : acc[2], 16);
+            const double s1 = __shfl_xor_sync(0xffffffffu, h16 ? acc[1] : acc[3], 16);
+            const double p0 = (h16 ? acc[2] : acc[0]) + s0, p1 = (h16 ? acc[3] : acc[1]) + s1;
+            double v = (h8 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h8 ? p0 : p1, 8);
+            for (int o = 4; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            const int k = (h16 ? 2 : 0) + (h8 ? 1 : 0);
+            if ((lane & 7) == 0 && r0 + k < mine)
+                bottom_put(base, a.o_cx + (rank + (r0 + k) * BOTTOM_CTAS) * (int)sizeof(T), (T)v);
+        }
+        cluster_arrive();
+        cluster_wait();
+    }
+    const int sq[3] = {a.seq.x, a.seq.y, a.seq.z};
+    for (int l = nl - 1; l >= 0; --l) {
+        const BottomLevel<T> &L = lv[l];
+        const T *xc = bottom_at<T>(sm, l + 1 < nl ? lv[l + 1].o_x : a.o_cx);
+        if (L.p1col) {
+            const int i = (w * BOTTOM_CTAS + rank) * 32 + lane;
+            if (i < L.n) {
+                const int c = bottom_at<int16_t>(sm, L.o_p1)[t];
+                bottom_put(base, L.o_x + i * (int)sizeof(T), c >= 0 ? xc[c] + T(0) : T(0));
+            }
+        } else {
+            bottom_spmv<T>(sm, base, L.v[BOTTOM_P], xc, L.o_x);
+        }
+        cluster_arrive();
+        cluster_wait();
+        for (int k = 0; k < 3 && sq[k] >= 0; ++k)
+            bottom_sweep<T>(sm, base, L.v[sq[k] == CF_F ? BOTTOM_AF : BOTTOM_AC], bottom_at<T>(sm, L.o_b), L.o_x);
+    }
+    for (int k = rank * BOTTOM_THREADS + t; k < a.n0; k += BOTTOM_CTAS * BOTTOM_THREADS)
+        a.x[k] = reinterpret_cast<const T *>(sm + a.o_x0)[k];
+}
+
+template <class T>
+void bottom_pack(const BottomLevel<T> *lv, int nl, int o_desc, int o_entries, int cap, int nz, const double *Ainv,
+                 int o_ainv, unsigned char *images, cudaStream_t s) {
+    k_bottom_pack<T><<<dim3(4 * nl, BOTTOM_CTAS), BOTTOM_THREADS, 0, s>>>(lv, nl, o_desc, o_entries, cap, nz, Ainv, o_ainv,
+                                                                          images);
     count_launch();
 }
-template void cycle_bottom<float>(const BottomLevel<float> *, int, const BottomCoarse<float> &, const int *,
-                                  cudaStream_t);
-template void cycle_bottom<double>(const BottomLevel<double> *, int, const BottomCoarse<double> &, const int *,
-                                   cudaStream_t);
+template void bottom_pack<float>(const BottomLevel<float> *, int, int, int, int, int, const double *, int, unsigned char *,
+                                 cudaStream_t);
+template void bottom_pack<double>(const BottomLevel<double> *, int, int, int, int, int, const double *, int,
+                                  unsigned char *, cudaStream_t);
+
+// whether the device can hold the bottom kernel's cluster
+template <class T>
+bool bottom_fits() {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(BOTTOM_CTAS);
+    cfg.blockDim = dim3(BOTTOM_THREADS);
+    cfg.dynamicSmemBytes = BOTTOM_SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = BOTTOM_CTAS;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    const bool ok = cudaFuncSetAttribute(k_cycle_bottom<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, BOTTOM_SMEM) ==
+                        cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&n, k_cycle_bottom<T>, &cfg) == cudaSuccess && n > 0;
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+template bool bottom_fits<float>();
+template bool bottom_fits<double>();
+
+template <class T>
+void cycle_bottom(const BottomArgs<T> &a, cudaStream_t s) {
+    launch_pdl(k_cycle_bottom<T>, BOTTOM_CTAS, BOTTOM_THREADS, BOTTOM_SMEM, s, a);
+    count_launch();
+}
+template void cycle_bottom<float>(const BottomArgs<float> &, cudaStream_t);
+template void cycle_bottom<double>(const BottomArgs<double> &, cudaStream_t);
 
 // the system of every 32-row block: that of its first row when its last row has the same one, else -1
 __global__ void k_blk_sys(int n, const int *__restrict__ seg, int nseg, int *__restrict__ blk_sys) {

@@ -232,26 +232,45 @@ void sell_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const
 // blocks of stopped systems are skipped
 template <class T>
 void p1_interp(int n, const int *p1col, const int *blk_sys, const uint8_t *run, const T *xc, T *x, cudaStream_t s);
-// the bottom of the V-cycle in one CTA (sell.cu): levels of at most BOTTOM_ROWS rows. A level: R restricts b to the
-// next level, P interpolates (sliced ELL, or the one-point column array p1col when set), AF / AC sweep the F / C
-// rows while crows / frows (nc / n - nc of them) are copied; the coarsest: x = Ainv b
+// the bottom of the V-cycle in one cluster of BOTTOM_CTAS CTAs (sell.cu): levels of at most BOTTOM_ROWS rows, at most
+// one row of a view per thread. A level: R restricts b to the next level, P interpolates (sliced ELL, or the one-point
+// column array p1col when set), AF / AC sweep the F / C rows; the coarsest: x = Ainv b. o_*: byte offsets in a CTA's
+// shared memory, which begins with the CTA's packed image of what the phases read (bottom_pack) and ends with the
+// levels' vectors. nloc: the CTA's slices of the view; o_val < 0: the entries did not fit and are read from col / val.
+constexpr int BOTTOM_R = 0, BOTTOM_P = 1, BOTTOM_AF = 2, BOTTOM_AC = 3;
+constexpr int BOTTOM_NOROW = 0xffff;
+template <class T> struct BottomView {
+    int nrows = 0, nloc = 0, o_ptr = 0, o_row = 0, o_dinv = 0, o_val = -1, o_col = -1, pad = 0;
+    const int *ptr = nullptr, *row = nullptr, *col = nullptr;
+    const T *val = nullptr, *dinv = nullptr;
+};
 template <class T> struct BottomLevel {
-    int n = 0, nc = 0;
-    SellView R, P, AF, AC;
+    int n = 0, o_b = 0, o_x = 0, o_p1 = 0;
     const int *p1col = nullptr;
-    const int *crows = nullptr, *frows = nullptr;
-    T *b = nullptr, *x[2] = {nullptr, nullptr};
+    BottomView<T> v[4];
 };
-template <class T> struct BottomCoarse {
-    int n = 0;
+template <class T> struct BottomArgs {
+    const unsigned char *img = nullptr;          // BOTTOM_CTAS images, BOTTOM_SMEM bytes apart
+    int nl = 0, n0 = 0, nc = 0;                  // bottom levels above the coarsest, rows of the first, of the coarsest
+    int o_desc = 0, o_b0 = 0, o_x0 = 0, o_cb = 0, o_cx = 0, o_ainv = -1;
     const double *Ainv = nullptr;
-    T *b = nullptr, *x = nullptr;
+    const T *b = nullptr;                        // the first level's right-hand side and result
+    T *x = nullptr;
+    int4 seq = {-1, -1, -1, 0};                  // the sweep targets (CF_F / CF_C, -1 ends)
 };
+// Whole V-cycle, one CTA reading L2 up to 1,024 rows -> one cluster up to 8,192 rows: 512^2 FD, FP32 one-point
+// 176 -> 151 us; 301^2 FD, FP64 lAIP 302 -> 228 us; 64^2 FD, FP64 lAIP 114 -> 95 us. A phase takes 0.7 us (a product) to
+// 1.1 us (a sweep), against 2.5 to 6 us as a kernel in the captured graph; 8,192 is one row per thread of the cluster.
+constexpr int BOTTOM_CTAS = 8;
 constexpr int BOTTOM_THREADS = 1024;
-constexpr int BOTTOM_ROWS = 1024;
-// lv: nl level descriptors in device memory; seq3: the sweep targets (CF_F / CF_C, -1 ends)
+constexpr int BOTTOM_ROWS = BOTTOM_CTAS * BOTTOM_THREADS;
+constexpr int BOTTOM_LEVELS = 25;                // more levels than this are not taken into the bottom
+constexpr int BOTTOM_SMEM = 224 * 1024;
 template <class T>
-void cycle_bottom(const BottomLevel<T> *lv, int nl, const BottomCoarse<T> &cz, const int *seq3, cudaStream_t s);
+void bottom_pack(const BottomLevel<T> *lv, int nl, int o_desc, int o_entries, int cap, int nz, const double *Ainv,
+                 int o_ainv, unsigned char *images, cudaStream_t s);
+template <class T> bool bottom_fits();           // also allows the kernel its shared memory: before cycle_bottom
+template <class T> void cycle_bottom(const BottomArgs<T> &a, cudaStream_t s);
 // the system of every 32-row block of a level (seg: first row of every system, nseg + 1 entries)
 void launch_blk_sys(int n, const int *seg, int nseg, int *blk_sys, cudaStream_t s);
 void launch_p1_cols(int n, const int *rp, const int *col, int *p1col, cudaStream_t s);
