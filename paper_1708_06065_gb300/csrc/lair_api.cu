@@ -478,10 +478,8 @@ static lair_status split_points(lair_handle *h, Temps &t, int l, int n, const Gr
         TRY(read_ints(h, mx, 3, deg));   // also keeps the host block list alive until its copy is done
         int nb = 8;
         while (nb < 2 * deg[2] + 1) nb *= 2;
-        const long long dl = 32 + (long long)deg[1] * (1 + deg[2]);
-        if (Bmax <= RSB_MAX_N && nb <= 256 && dl <= RSB_MAX_DIRTY &&
-            rsb_smem_bytes(Bmax, nb, (int)dl) <= (size_t)200 * 1024) {
-            CU(launch_rs_bucket(bd, (int)blocks.size(), Bmax, nb, (int)dl, deg[0], Scf, STcf, cf, h->status, h->s));
+        if (Bmax <= RSB_MAX_N && nb <= 256 && rsb_smem_bytes(Bmax, nb) <= (size_t)200 * 1024) {
+            CU(launch_rs_bucket(bd, (int)blocks.size(), Bmax, nb, deg[0], Scf, STcf, cf, h->status, h->s));
         } else {
             CU(launch_rs(n, bd, (int)blocks.size(), Bmax, deg[0], Scf, STcf, cf, h->status, h->s));
         }

@@ -638,12 +638,18 @@ __global__ void __launch_bounds__(32) k_rs_count(const int2 *__restrict__ blocks
 }
 
 // per block: the in-block entries of S (for staging), and the largest in-block row lengths of S and ST;
-// out[0..2] take the maxima over all blocks
-__global__ void __launch_bounds__(32) k_rs_degrees(const int2 *__restrict__ blocks, Graph S, Graph ST,
-                                                   int *__restrict__ out) {
+// out[0..2] take the maxima over all blocks. Bound by the latency of its row reads, so a CTA of eight warps per
+// block (64^2 FD, one block of 4,096 points: 141 us with one warp, 14 us).
+constexpr int RS_DEG_THREADS = 256;
+
+__global__ void __launch_bounds__(RS_DEG_THREADS) k_rs_degrees(const int2 *__restrict__ blocks, Graph S, Graph ST,
+                                                               int *__restrict__ out) {
+    __shared__ int total;
     const int b0 = blocks[blockIdx.x].x, b1 = blocks[blockIdx.x].y;
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
     int c = 0, ms = 0, mt = 0;
-    for (int i = b0 + threadIdx.x; i < b1; i += 32) {
+    for (int i = b0 + threadIdx.x; i < b1; i += RS_DEG_THREADS) {
         int ds = 0, dt = 0;
         for (int p = S.rp[i]; p < S.rp[i + 1]; ++p) ds += (S.col[p] >= b0 && S.col[p] < b1);
         for (int p = ST.rp[i]; p < ST.rp[i + 1]; ++p) dt += (ST.col[p] >= b0 && ST.col[p] < b1);
@@ -654,11 +660,13 @@ __global__ void __launch_bounds__(32) k_rs_degrees(const int2 *__restrict__ bloc
     c = __reduce_add_sync(0xffffffffu, c);
     ms = __reduce_max_sync(0xffffffffu, ms);
     mt = __reduce_max_sync(0xffffffffu, mt);
-    if (threadIdx.x == 0) {
-        atomicMax(&out[0], c);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&total, c);
         atomicMax(&out[1], ms);
         atomicMax(&out[2], mt);
     }
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(&out[0], total);
 }
 
 // -------------------------------------------------------------------------------------
@@ -666,32 +674,34 @@ __global__ void __launch_bounds__(32) k_rs_degrees(const int2 *__restrict__ bloc
 // stays below nb buckets (lambda_k <= 2 |ST_k n block|: it starts at the in-block count and each
 // dependant adds one when it becomes F). Bucket b is a bitmap over the block of the undecided
 // points with lambda = b, so the point to take (largest lambda, then smallest index) is the lowest
-// set bit of the highest non-empty bucket. The graphs are read through the cache; shared memory
-// holds only the buckets and per-point bytes, so many blocks run on one SM at once. A step:
+// set bit of the highest non-empty bucket. A step:
 //   1. find i, which becomes C;
 //   2. its undecided in-block dependants (ST_i) become F and leave their buckets;
 //   3. lambda_k += 1 for undecided in-block k in S_j of every new F point j and lambda_k -= 1 for
-//      undecided in-block k in S_i (byte atomics on lambda; each changed k is listed once);
-//   4. every listed k moves from the bucket of its previous lambda to that of its new one.
+//      undecided in-block k in S_i; every such k moves to the bucket of its new lambda.
 // The sequence of points taken is the one of the tree version above (and of the oracle).
+//
+// The steps depend on one another, so what bounds the kernel is the chain of shared-memory latencies of one
+// step. One warp runs them: the rows of step 3 (that of i and those of the new F points) are read four at a time
+// by eight lanes each, and the changes of one point that several lanes hold are summed with a warp match, so a
+// step is one pass of that chain however many neighbours it touches. (Walking S_j entry by entry in the lane
+// that made j an F point, with shared-memory atomics that return and a list of changed points: 1.4 us a step.)
+// The other warps of the CTA only help to set the block up.
 // -------------------------------------------------------------------------------------
 struct RsbLayout {
     int W;                                // bitmap words per bucket (a multiple of 128)
-    size_t bm, cnt, dflag, dlist, lam, bkt, cf, total;   // byte offsets in dynamic shared memory
+    size_t bm, cnt, lam, cf, total;       // byte offsets in dynamic shared memory
 };
 
 __host__ __device__ inline size_t rsb_round16(size_t b) { return (b + 15) & ~(size_t)15; }
 
-__host__ __device__ inline RsbLayout rsb_layout(int n, int nb, int dl) {
+__host__ __device__ inline RsbLayout rsb_layout(int n, int nb) {
     RsbLayout L;
     L.W = (((n + 31) / 32) + 127) / 128 * 128;
     size_t o = 0;
     L.bm = o;    o += rsb_round16((size_t)nb * L.W * sizeof(unsigned));
     L.cnt = o;   o += rsb_round16((size_t)nb * sizeof(int));
-    L.dflag = o; o += rsb_round16((size_t)L.W * sizeof(unsigned));
-    L.dlist = o; o += rsb_round16((size_t)dl * sizeof(int));
-    L.lam = o;   o += rsb_round16((size_t)n);          // one byte per point, updated by 32-bit atomics
-    L.bkt = o;   o += rsb_round16((size_t)n);
+    L.lam = o;   o += rsb_round16((size_t)n);
     L.cf = o;    o += rsb_round16((size_t)n);
     L.total = o;
     return L;
@@ -700,26 +710,77 @@ __host__ __device__ inline RsbLayout rsb_layout(int n, int nb, int dl) {
 struct RsbShared {
     unsigned *bm;      // nb bitmaps of W words
     int *cnt;          // points per bucket
-    unsigned *dflag;   // listed in this step
-    int *dlist;        // points whose lambda changed in this step
-    unsigned *lamw;    // byte k: lambda_k
-    uint8_t *bkt;      // the bucket that holds k
+    uint8_t *lam;      // lambda_k: the bucket that holds an undecided k
     int8_t *cf;
-    int *ndirty;
 };
 
-// the steps of the bucket-queue first pass over in-block views of S and ST (local indices)
+// Step 3 for one set of rows: lane l holds the row [rb, re) of S (empty: no row) whose entries change by +1, or by -1
+// for the row of lane minus (the C point; -1: none). Returns the largest new lambda.
 template <class V>
-__device__ void rsb_steps(int n, int nb, int W, int dl, int top, const V &Sv, const V &STv, const RsbShared &q,
-                          int *status) {
-    const unsigned lane = threadIdx.x;
+__device__ __forceinline__ int rsb_touch(int nb, int W, const V &Sv, const RsbShared &q, int rb, int re, int minus,
+                                         int *status) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned rows = __ballot_sync(FULL, rb < re);
+    int hi = 0;
+    while (rows) {
+        // the next four rows, eight lanes each
+        int src = -1;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const int b = rows ? __ffs(rows) - 1 : -1;
+            if ((lane >> 3) == g) src = b;
+            rows &= rows - 1;   // 0 stays 0
+        }
+        int r = __shfl_sync(FULL, rb, src < 0 ? 0 : src) + (lane & 7);
+        const int e = __shfl_sync(FULL, re, src < 0 ? 0 : src);
+        const bool dec = src == minus;
+        bool in = src >= 0 && r < e;
+        do {
+            int k = -1;
+            if (in) {
+                k = Sv.at(r);
+                if (k >= 0 && q.cf[k] != CF_U) k = -1;
+            }
+            // lanes that hold the same point: the lowest of them applies the sum of their changes
+            const unsigned same = __match_any_sync(FULL, k);
+            const unsigned down = __ballot_sync(FULL, dec);
+            if (k >= 0 && lane == __ffs(same) - 1) {
+                const int d = __popc(same & ~down) - __popc(same & down);
+                if (d != 0) {
+                    const int ob = q.lam[k], nl = ob + d;
+                    if (nl < 0 || nl >= nb) {   // the host sized nb above every reachable lambda
+                        set_status(status, LAIR_ERR_ARENA_OVERFLOW);
+                    } else {
+                        const unsigned bit = 1u << (k & 31);
+                        atomicAnd(&q.bm[ob * W + (k >> 5)], ~bit);
+                        atomicOr(&q.bm[nl * W + (k >> 5)], bit);
+                        atomicSub(&q.cnt[ob], 1);
+                        atomicAdd(&q.cnt[nl], 1);
+                        q.lam[k] = (uint8_t)nl;
+                        hi = max(hi, nl);
+                    }
+                }
+            }
+            __syncwarp();
+            r += 8;
+            in = src >= 0 && r < e;
+        } while (__any_sync(FULL, in));
+    }
+    return hi;
+}
+
+// the steps of the bucket-queue first pass over in-block views of S and ST (local indices), one warp
+template <class V>
+__device__ void rsb_steps(int n, int nb, int W, int top, const V &Sv, const V &STv, const RsbShared &q, int *status) {
+    const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     const int per = W / 32;                    // bitmap words scanned by each lane (4 or more, contiguous)
     for (int step = 0; step <= n; ++step) {
         // 1. the highest non-empty bucket at or below top, then its lowest set bit
         int b = -1;
         for (int t0 = top; t0 >= 0; t0 -= 32) {
-            const int c = t0 - (int)lane;
+            const int c = t0 - lane;
             const unsigned m = __ballot_sync(FULL, c >= 0 && q.cnt[c] > 0);
             if (m) {
                 b = t0 - (__ffs(m) - 1);
@@ -744,133 +805,163 @@ __device__ void rsb_steps(int n, int nb, int W, int dl, int top, const V &Sv, co
             break;
         }
         const int src = __ffs(fm) - 1;
-        fw = __shfl_sync(FULL, fw, src) + src * per;
-        fv = __shfl_sync(FULL, fv, src);
-        const int li = 32 * fw + __ffs(fv) - 1;
+        const int li = __shfl_sync(FULL, 32 * (fw + lane * per) + __ffs(fv) - 1, src);
         // 2. li becomes C; its undecided in-block dependants become F (new in this step)
+        const int sb = STv.beg(li), se = STv.end(li);
+        const int ib = Sv.beg(li), ie = Sv.end(li);
         if (lane == 0) {
             q.cf[li] = CF_C;
             atomicAnd(&q.bm[b * W + (li >> 5)], ~(1u << (li & 31)));
             atomicSub(&q.cnt[b], 1);
         }
-        const int sb = STv.beg(li), se = STv.end(li);
-        for (int p = sb + (int)lane; p < se; p += 32) {
-            const int j = STv.at(p);
-            if (j >= 0 && q.cf[j] == CF_U) {
-                q.cf[j] = CF_NEWF;
-                const int bj = q.bkt[j];
-                atomicAnd(&q.bm[bj * W + (j >> 5)], ~(1u << (j & 31)));
-                atomicSub(&q.cnt[bj], 1);
-            }
-        }
-        __syncwarp();
-        // 3. lambda updates; the first touch of a point lists it
-        auto touch = [&](int k, bool inc) {
-            const unsigned sh = 8u * (unsigned)(k & 3);
-            atomicAdd(&q.lamw[k >> 2], inc ? (1u << sh) : (0u - (1u << sh)));
-            const unsigned bit = 1u << (k & 31);
-            if (!(atomicOr(&q.dflag[k >> 5], bit) & bit)) {
-                const int pos = atomicAdd(q.ndirty, 1);
-                if (pos < dl) q.dlist[pos] = k;
-                else set_status(status, LAIR_ERR_ARENA_OVERFLOW);
-            }
+        auto leave = [&](int j) {
+            const int bj = q.lam[j];
+            atomicAnd(&q.bm[bj * W + (j >> 5)], ~(1u << (j & 31)));
+            atomicSub(&q.cnt[bj], 1);
         };
-        for (int p = sb + (int)lane; p < se; p += 32) {
-            const int j = STv.at(p);
-            if (j < 0 || q.cf[j] != CF_NEWF) continue;
-            for (int r = Sv.beg(j); r < Sv.end(j); ++r) {
-                const int k = Sv.at(r);
-                if (k >= 0 && q.cf[k] == CF_U) touch(k, true);
-            }
-        }
-        for (int r = Sv.beg(li) + (int)lane; r < Sv.end(li); r += 32) {
-            const int k = Sv.at(r);
-            if (k >= 0 && q.cf[k] == CF_U) touch(k, false);
-        }
-        __syncwarp();
-        // 4. listed points change bucket
-        const int nd = min(*q.ndirty, dl);
         int hi = 0;
-        for (int d = lane; d < nd; d += 32) {
-            const int k = q.dlist[d];
-            const unsigned bit = 1u << (k & 31);
-            atomicAnd(&q.dflag[k >> 5], ~bit);
-            const int lam = (int)((q.lamw[k >> 2] >> (8 * (k & 3))) & 0xFFu);
-            const int ob = q.bkt[k];
-            if (lam == ob) continue;
-            if (lam >= nb) {
-                set_status(status, LAIR_ERR_ARENA_OVERFLOW);
-                continue;
+        if (se - sb < 32) {
+            // lanes 0 .. 30: one dependant each; lane 31: the row of li itself
+            int rb = 0, re = 0;
+            if (lane < se - sb) {
+                const int j = STv.at(sb + lane);
+                if (j >= 0) {
+                    rb = Sv.beg(j);
+                    re = Sv.end(j);
+                    if (q.cf[j] == CF_U) {
+                        q.cf[j] = CF_F;
+                        leave(j);
+                    } else {
+                        re = rb;
+                    }
+                }
+            } else if (lane == 31) {
+                rb = ib;
+                re = ie;
             }
-            atomicAnd(&q.bm[ob * W + (k >> 5)], ~bit);
-            atomicOr(&q.bm[lam * W + (k >> 5)], bit);
-            atomicSub(&q.cnt[ob], 1);
-            atomicAdd(&q.cnt[lam], 1);
-            q.bkt[k] = (uint8_t)lam;
-            hi = max(hi, lam);
+            __syncwarp();
+            hi = rsb_touch(nb, W, Sv, q, rb, re, 31, status);
+        } else {
+            for (int p = sb + lane; p < se; p += 32) {
+                const int j = STv.at(p);
+                if (j >= 0 && q.cf[j] == CF_U) {
+                    q.cf[j] = CF_NEWF;
+                    leave(j);
+                }
+            }
+            __syncwarp();
+            hi = rsb_touch(nb, W, Sv, q, lane == 31 ? ib : 0, lane == 31 ? ie : 0, 31, status);
+            for (int p0 = sb; p0 < se; p0 += 32) {
+                const int j = p0 + lane < se ? STv.at(p0 + lane) : -1;
+                const bool isnew = j >= 0 && q.cf[j] == CF_NEWF;
+                hi = max(hi, rsb_touch(nb, W, Sv, q, isnew ? Sv.beg(j) : 0, isnew ? Sv.end(j) : 0, -2, status));
+            }
+            for (int p = sb + lane; p < se; p += 32) {
+                const int j = STv.at(p);
+                if (j >= 0 && q.cf[j] == CF_NEWF) q.cf[j] = CF_F;
+            }
+            __syncwarp();
         }
         top = max(top, (int)__reduce_max_sync(FULL, (unsigned)hi));
-        __syncwarp();
-        if (lane == 0) *q.ndirty = 0;
-        for (int p = sb + (int)lane; p < se; p += 32) {
-            const int j = STv.at(p);
-            if (j >= 0 && q.cf[j] == CF_NEWF) q.cf[j] = CF_F;
-        }
-        __syncwarp();
     }
+}
+
+// copy the in-block part of graph G (rows b0..b1-1) into shared memory, all threads of the CTA; false if it does not
+// fit in cap entries (nothing is used then)
+__device__ bool rsb_stage(const Graph &G, int b0, int b1, uint16_t *rp, uint16_t *col, size_t cap_entries) {
+    __shared__ int wsum[32], tot;
+    const int t = threadIdx.x, T = blockDim.x, lane = t & 31, w = t >> 5, n = b1 - b0;
+    for (int li = t; li < n; li += T) {
+        int c = 0;
+        for (int p = G.rp[b0 + li]; p < G.rp[b0 + li + 1]; ++p) c += (G.col[p] >= b0 && G.col[p] < b1);
+        rp[li] = (uint16_t)c;
+    }
+    __syncthreads();
+    const int chunk = (n + T - 1) / T, r0 = min(n, t * chunk), r1 = min(n, r0 + chunk);
+    int mine = 0;
+    for (int li = r0; li < r1; ++li) mine += rp[li];
+    int incl = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    if (t == 0) {
+        int s = 0;
+        for (int k = 0; k < T / 32; ++k) {
+            const int c = wsum[k];
+            wsum[k] = s;
+            s += c;
+        }
+        tot = s;
+    }
+    __syncthreads();
+    const int total = tot;
+    if ((size_t)total > cap_entries || total > 65535) return false;
+    int run = wsum[w] + incl - mine;
+    for (int li = r0; li < r1; ++li) {
+        const int c = rp[li];
+        rp[li] = (uint16_t)run;
+        run += c;
+    }
+    if (t == 0) rp[n] = (uint16_t)total;
+    __syncthreads();
+    for (int li = t; li < n; li += T) {
+        int q = rp[li];
+        for (int p = G.rp[b0 + li]; p < G.rp[b0 + li + 1]; ++p) {
+            const int j = G.col[p];
+            if (j >= b0 && j < b1) col[q++] = (uint16_t)(j - b0);
+        }
+    }
+    __syncthreads();
+    return true;
 }
 
 // smem_bytes: the bucket layout of the largest block, plus (stage != 0) room to stage both in-block graphs
 // (uint16 row offsets and columns) so that each step reads shared memory only. Staging pays when the level
 // has at most one block per SM; with more blocks it costs occupancy, which hides more of each step's
 // latency than the staging saves (measured), and the graphs are read through the cache.
-__global__ void __launch_bounds__(32) k_rs_bucket(const int2 *__restrict__ blocks, Graph S, Graph ST, int nb, int dl,
-                                                  int8_t *__restrict__ cf_out, int *status, int stage,
-                                                  int smem_bytes) {
+__global__ void __launch_bounds__(RSB_THREADS) k_rs_bucket(const int2 *__restrict__ blocks, Graph S, Graph ST, int nb,
+                                                           int8_t *__restrict__ cf_out, int *status, int stage,
+                                                           int smem_bytes) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int ndirty;
+    __shared__ int top_s;
     const int b0 = blocks[blockIdx.x].x, b1 = blocks[blockIdx.x].y;
-    const int n = b1 - b0;
-    const RsbLayout Lo = rsb_layout(n, nb, dl);
+    const int n = b1 - b0, t = threadIdx.x, T = blockDim.x;
+    const RsbLayout Lo = rsb_layout(n, nb);
     const int W = Lo.W;
     RsbShared q;
     q.bm = reinterpret_cast<unsigned *>(smem + Lo.bm);
     q.cnt = reinterpret_cast<int *>(smem + Lo.cnt);
-    q.dflag = reinterpret_cast<unsigned *>(smem + Lo.dflag);
-    q.dlist = reinterpret_cast<int *>(smem + Lo.dlist);
-    q.lamw = reinterpret_cast<unsigned *>(smem + Lo.lam);
-    q.bkt = smem + Lo.bkt;
+    q.lam = smem + Lo.lam;
     q.cf = reinterpret_cast<int8_t *>(smem + Lo.cf);
-    q.ndirty = &ndirty;
-    const unsigned lane = threadIdx.x;
 
-    for (int e = lane; e < nb * W; e += 32) q.bm[e] = 0u;
-    for (int e = lane; e < nb; e += 32) q.cnt[e] = 0;
-    for (int e = lane; e < W; e += 32) q.dflag[e] = 0u;
-    for (int e = lane; e < (n + 3) / 4; e += 32) q.lamw[e] = 0u;
-    if (lane == 0) ndirty = 0;
-    __syncwarp();
+    for (int e = t; e < nb * W; e += T) q.bm[e] = 0u;
+    for (int e = t; e < nb; e += T) q.cnt[e] = 0;
+    if (t == 0) top_s = 0;
+    __syncthreads();
     int top = 0;
-    for (int li = lane; li < n; li += 32) {
+    for (int li = t; li < n; li += T) {
         const int i = b0 + li;
         int lam = 0;
         for (int p = ST.rp[i]; p < ST.rp[i + 1]; ++p) lam += (ST.col[p] >= b0 && ST.col[p] < b1);
         const bool iso = (S.rp[i + 1] == S.rp[i]) && (ST.rp[i + 1] == ST.rp[i]);
         q.cf[li] = iso ? CF_F : CF_U;
-        q.bkt[li] = 0;
+        q.lam[li] = 0;
         if (iso) continue;
         if (lam >= nb) {                       // the host sized nb above every reachable lambda
             set_status(status, LAIR_ERR_ARENA_OVERFLOW);
             lam = nb - 1;
         }
-        atomicAdd(&q.lamw[li >> 2], (unsigned)lam << (8 * (li & 3)));
-        q.bkt[li] = (uint8_t)lam;
+        q.lam[li] = (uint8_t)lam;
         atomicOr(&q.bm[lam * W + (li >> 5)], 1u << (li & 31));
         atomicAdd(&q.cnt[lam], 1);
         top = max(top, lam);
     }
     top = (int)__reduce_max_sync(0xffffffffu, (unsigned)top);
-    __syncwarp();
+    if ((t & 31) == 0) atomicMax(&top_s, top);
+    __syncthreads();
     bool staged = false;
     uint16_t *srp = reinterpret_cast<uint16_t *>(smem + Lo.total);
     uint16_t *strp = srp + (n + 1);
@@ -878,24 +969,28 @@ __global__ void __launch_bounds__(32) k_rs_bucket(const int2 *__restrict__ block
     if (stage) {
         const size_t used = (size_t)(reinterpret_cast<unsigned char *>(scol) - smem);
         const size_t cap = used < (size_t)smem_bytes ? ((size_t)smem_bytes - used) / (2 * sizeof(uint16_t)) : 0;
-        staged = rs_stage(S, b0, b1, srp, scol, cap);
-        if (staged) staged = rs_stage(ST, b0, b1, strp, scol + srp[n], cap);
+        staged = rsb_stage(S, b0, b1, srp, scol, cap);
+        if (staged) staged = rsb_stage(ST, b0, b1, strp, scol + srp[n], cap);
     }
-    if (staged) {
-        StagedView vs{srp, scol}, vt{strp, scol + srp[n]};
-        rsb_steps(n, nb, W, dl, top, vs, vt, q, status);
-    } else {
-        GlobalView vs{S.rp, S.col, b0, b1}, vt{ST.rp, ST.col, b0, b1};
-        rsb_steps(n, nb, W, dl, top, vs, vt, q, status);
+    if (t < 32) {
+        top = top_s;
+        if (staged) {
+            StagedView vs{srp, scol}, vt{strp, scol + srp[n]};
+            rsb_steps(n, nb, W, top, vs, vt, q, status);
+        } else {
+            GlobalView vs{S.rp, S.col, b0, b1}, vt{ST.rp, ST.col, b0, b1};
+            rsb_steps(n, nb, W, top, vs, vt, q, status);
+        }
     }
-    for (int li = lane; li < n; li += 32) {
+    __syncthreads();
+    for (int li = t; li < n; li += T) {
         const int8_t c = q.cf[li];
         if (c != CF_C && c != CF_F) set_status(status, LAIR_ERR_DEVICE_TIMEOUT);
         cf_out[b0 + li] = c;
     }
 }
 
-size_t rsb_smem_bytes(int n, int nb, int dl) { return rsb_layout(n, nb, dl).total; }
+size_t rsb_smem_bytes(int n, int nb) { return rsb_layout(n, nb).total; }
 
 // the bytes to stage both in-block graphs of the fullest block as well
 static size_t rsb_stage_bytes(int n, int max_inblock) {
@@ -1274,13 +1369,13 @@ void launch_rs_count(const int2 *blocks, int nblocks, const Graph &S, int *maxcn
 }
 
 void launch_rs_degrees(const int2 *blocks, int nblocks, const Graph &S, const Graph &ST, int *out, cudaStream_t s) {
-    k_rs_degrees<<<nblocks, 32, 0, s>>>(blocks, S, ST, out);
+    k_rs_degrees<<<nblocks, RS_DEG_THREADS, 0, s>>>(blocks, S, ST, out);
     count_launch();
 }
 
-cudaError_t launch_rs_bucket(const int2 *blocks, int nblocks, int Bmax, int nb, int dl, int max_inblock,
-                             const Graph &S, const Graph &ST, int8_t *cf, int *status, cudaStream_t s) {
-    size_t bytes = rsb_smem_bytes(Bmax, nb, dl);
+cudaError_t launch_rs_bucket(const int2 *blocks, int nblocks, int Bmax, int nb, int max_inblock, const Graph &S,
+                             const Graph &ST, int8_t *cf, int *status, cudaStream_t s) {
+    size_t bytes = rsb_smem_bytes(Bmax, nb);
     int stage = 0;
     if (nblocks <= device_sms()) {
         const size_t want = bytes + rsb_stage_bytes(Bmax, max_inblock);
@@ -1289,7 +1384,9 @@ cudaError_t launch_rs_bucket(const int2 *blocks, int nblocks, int Bmax, int nb, 
     }
     cudaError_t e = cudaFuncSetAttribute(k_rs_bucket, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    k_rs_bucket<<<nblocks, 32, bytes, s>>>(blocks, S, ST, nb, dl, cf, status, stage, (int)bytes);
+    // a few warps to set the block up; many blocks on an SM need no more than two each
+    const int tb = stage ? RSB_THREADS : 64;
+    k_rs_bucket<<<nblocks, tb, bytes, s>>>(blocks, S, ST, nb, cf, status, stage, (int)bytes);
     count_launch();
     return cudaGetLastError();
 }
