@@ -936,6 +936,7 @@ static lair_status build_sells(lair_handle *h, Hier &H, std::vector<SellPlan> &p
             if (p.nrows <= 0 || (p.fp32 ? 0 : 1) != g) continue;
             SellView &v = *p.v;
             v.nrows = p.nrows;
+            v.long_rows = (long long)p.M->nnz > (long long)WAVE_SHORT * p.M->nr;
             TRY(dalloc(h, &v.row, (size_t)p.nrows));
             const int nsl = (p.nrows + 31) / 32;
             SellDesc d{};
@@ -1273,7 +1274,7 @@ static lair_status autotune_level(lair_handle *h, Hier &H, int l, cudaEvent_t e0
     };
     for (int kind = 0; kind < 4; ++kind) {
         SellView &v = *jobs[kind].v;
-        if (v.nrows < TUNE_MIN_ROWS) continue;
+        if (v.nrows < TUNE_MIN_ROWS || v.nrows <= one_wave_rows<T>()) continue;   // one-wave views have one schedule
         const TuneKey key{dev, kind, (int)sizeof(T), (int)std::floor(4.0 * std::log2((double)v.nrows)),
                           (int)std::lround(jobs[kind].len)};
         {
@@ -1342,18 +1343,16 @@ static lair_status autotune_views(lair_handle *h, Hier &H) {
     return st;
 }
 
-// The smallest levels (at most BOTTOM_ROWS rows, below the finest, at least one besides the coarsest) run in the
-// one-cluster bottom kernel. Their descriptors are written here in the cycle's precision: the offsets in a CTA's shared
+// The smallest levels (at most BOTTOM_ROWS rows and few enough entries, below the finest, at least one besides the
+// coarsest) run in the bottom kernel. Their descriptors are written here in the cycle's precision: the offsets in shared
 // memory of the lists, the coarsest inverse and the vectors, whose sizes the host knows; what is left takes view
 // entries (bottom_pack). A bottom whose lists and vectors alone do not fit starts one level further down. The views
-// that the descriptors point to live as long as the hierarchy; a refresh refills them in place and packs the images
+// that the descriptors point to live as long as the hierarchy; a refresh refills them in place and packs the image
 // again.
 template <class T>
 static void pack_bottom(lair_handle *h, Hier &H) {
-    const Level &Z = H.lev.back();
     bottom_pack<T>(static_cast<const BottomLevel<T> *>(H.bottom_desc), (int)H.lev.size() - 1 - H.bottom_first,
-                   H.bottom_o.desc, H.bottom_o.entries, H.bottom_o.top, Z.A.nr, Z.Ainv, H.bottom_o.ainv, H.bottom_img,
-                   h->s);
+                   H.bottom_o.desc, H.bottom_o.entries, H.bottom_o.top, H.bottom_img, h->s);
 }
 
 template <class T>
@@ -1364,7 +1363,7 @@ static lair_status prepare_bottom(lair_handle *h, Hier &H) {
     if (h->o.nodal > 1 || nl < 3 || H.lev[nl - 1].A.nr > 512 || !bottom_fits<T>()) return LAIR_OK;
     int first = -1;
     for (int l = 1; l <= nl - 2 && first < 0; ++l)
-        if (H.lev[l].A.nr <= BOTTOM_ROWS && nl - 1 - l <= BOTTOM_LEVELS) first = l;
+        if (H.lev[l].A.nr <= BOTTOM_ROWS && H.lev[l].A.nnz <= bottom_entries<T>() && nl - 1 - l <= BOTTOM_LEVELS) first = l;
     if (first < 0) return LAIR_OK;
     auto &o = H.bottom_o;
     std::vector<BottomLevel<T>> d;
@@ -1377,7 +1376,6 @@ static lair_status prepare_bottom(lair_handle *h, Hier &H) {
             return p;
         };
         auto take_vec = [&](size_t bytes) { return top -= (int)((bytes + 15) & ~(size_t)15); };
-        auto slices = [](int rows) { return ((rows + 31) / 32 + BOTTOM_CTAS - 1) / BOTTOM_CTAS; };   // of one CTA
         o.desc = take(sizeof(BottomLevel<T>) * d.size());
         for (int i = 0; i < (int)d.size(); ++i) {
             Level &L = H.lev[first + i];
@@ -1387,7 +1385,7 @@ static lair_status prepare_bottom(lair_handle *h, Hier &H) {
             t.o_x = take_vec(sizeof(T) * t.n);
             if (h->o.interp == LAIR_P_ONEPOINT) {
                 t.p1col = L.p1col;
-                t.o_p1 = take(sizeof(int16_t) * 32 * slices(t.n));
+                t.o_p1 = take(sizeof(int16_t) * t.n);
             }
             const SellView *src[4];
             src[BOTTOM_R] = &L.Rv;
@@ -1404,16 +1402,17 @@ static lair_status prepare_bottom(lair_handle *h, Hier &H) {
                 v.val = static_cast<const T *>(s.val);
                 v.dinv = static_cast<const T *>(s.dinv);
                 if (v.nrows <= 0) continue;
-                v.o_ptr = take(sizeof(int2) * slices(v.nrows));
-                v.o_row = take(sizeof(uint16_t) * 32 * slices(v.nrows));
-                if (v.dinv) v.o_dinv = take(sizeof(T) * 32 * slices(v.nrows));
+                v.o_ptr = take(sizeof(int2) * ((v.nrows + 31) / 32));
+                v.o_row = take(sizeof(uint16_t) * v.nrows);
+                if (v.dinv) v.o_dinv = take(sizeof(T) * v.nrows);
             }
         }
         const int nz = H.lev[nl - 1].A.nr;
         o.cb = take_vec(sizeof(T) * nz);
         o.cx = take_vec(sizeof(T) * nz);
+        // the inverse's rows of a CTA stand before the vectors: the image, which ends before them, does not hold them
         const size_t inv = sizeof(double) * (size_t)((nz + BOTTOM_CTAS - 1) / BOTTOM_CTAS) * nz;
-        o.ainv = at + (long long)inv + 64 <= top ? take(inv) : -1;
+        o.ainv = at + (long long)inv + 64 <= top ? take_vec(inv) : -1;
         o.entries = (at + 63) & ~63;
         o.top = top;
         if (o.entries <= top) break;
@@ -1424,7 +1423,7 @@ static lair_status prepare_bottom(lair_handle *h, Hier &H) {
     const size_t bytes = sizeof(BottomLevel<T>) * d.size();
     char *desc = nullptr;
     TRY(dalloc(h, &desc, bytes));
-    TRY(dalloc(h, &H.bottom_img, (size_t)BOTTOM_SMEM * BOTTOM_CTAS));
+    TRY(dalloc(h, &H.bottom_img, (size_t)BOTTOM_SMEM));
     CU(cudaMemcpyAsync(desc, d.data(), bytes, cudaMemcpyHostToDevice, h->s));
     // (a copy from pageable memory is staged before cudaMemcpyAsync returns, so d may go)
     H.bottom_desc = desc;

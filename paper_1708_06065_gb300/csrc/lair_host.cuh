@@ -71,11 +71,11 @@ struct Hier {
     double setup_ms = 0.0;
     // the sliced-ELL fill descriptors of all views (device), kept so that a refresh refills the views in place
     SellDesc *sell_desc = nullptr;
-    // the bottom of the cycle in one cluster: levels bottom_first .. coarsest (-1: a kernel per phase everywhere);
-    // bottom_desc holds their BottomLevel descriptors in the cycle's precision, bottom_img the packed images that the
-    // kernel's CTAs copy to shared memory (packed again by a refresh); byte offsets of the descriptors, of the
-    // coarsest inverse's rows (-1: not in the image), of the entries, of the first byte taken by vectors, and of the
-    // vectors that the kernel's arguments name
+    // the bottom of the cycle in one launch: levels bottom_first .. coarsest (-1: a kernel per phase everywhere);
+    // bottom_desc holds their BottomLevel descriptors in the cycle's precision, bottom_img the packed image that the
+    // kernel copies to shared memory (packed again by a refresh); byte offsets of the descriptors, of the coarsest
+    // inverse's rows (-1: not in shared memory), of the entries, of the first byte taken by vectors, and of the vectors
+    // that the kernel's arguments name
     int bottom_first = -1;
     void *bottom_desc = nullptr;
     unsigned char *bottom_img = nullptr;

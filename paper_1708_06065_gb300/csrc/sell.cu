@@ -346,6 +346,108 @@ __global__ void __launch_bounds__(256) k_sell_sweep(SellView v, const int *__res
     }
 }
 
+// The same product and sweep for views whose rows fit on the GPU in one wave. There a launch is bound by its chain of
+// dependent loads -- slice offset, columns, gathered x, then row and b -- and by the launch itself, not by bandwidth.
+// So a thread has one row and brings everything that does not depend on the previous kernel of the cycle (offsets,
+// the first NB values and columns, the Jacobi diagonal, the row's index) into registers before it waits for that
+// kernel; then come NB gathers at once and the sum, in column order as above. x, b and xo are plain pointers: their
+// loads must stay behind the wait. More registers and fewer resident warps than the kernels above, which is why
+// larger views do not take it (one_wave_rows).
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class T, int NB>
+struct RowHead {
+    int base = 0, len = 0, i = -1;
+    int c[NB];
+    T w[NB];
+    // row slot u of the view (u < 32 * slices); a slice of a stopped system has no row, or a row without entries when
+    // its rows are to be written as 0
+    __device__ __forceinline__ void load(const SellView &v, int u, int nrows) {
+        const int sl = u >> 5, lane = u & 31;
+        bool on = true, zero = false;
+        if (v.run) {
+            const int q = v.slice_sys[sl];
+            on = q < 0 || v.run[q];
+            zero = !on && v.zero_stopped;
+        }
+        if (on) {
+            const int a = __ldg(v.slice_ptr + sl);
+            base = a + lane;
+            len = (__ldg(v.slice_ptr + sl + 1) - a) >> 5;
+        }
+        if ((on || zero) && u < nrows) i = __ldg(v.row + u);
+        const T *val = static_cast<const T *>(v.val);
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            c[k] = k < len ? __ldg(v.col + base + 32 * k) : 0;
+            w[k] = k < len ? __ldg(val + base + 32 * k) : T(0);
+        }
+    }
+    __device__ __forceinline__ T sum(const SellView &v, const T *x) const {
+        T acc = T(0);
+        {
+            T xv[NB];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) xv[k] = k < len ? x[c[k]] : T(0);
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+                if (k < len) acc = fma(w[k], xv[k], acc);
+        }
+        const T *val = static_cast<const T *>(v.val);
+        for (int j = NB; j < len; j += NB) {
+            int cc[NB];
+            T ww[NB];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                cc[k] = j + k < len ? __ldg(v.col + base + 32 * (j + k)) : 0;
+                ww[k] = j + k < len ? __ldg(val + base + 32 * (j + k)) : T(0);
+            }
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+                if (j + k < len) acc = fma(ww[k], x[cc[k]], acc);
+        }
+        return acc;
+    }
+};
+
+constexpr int WAVE_THREADS = 128;
+
+template <class T, int NB>
+__global__ void __launch_bounds__(WAVE_THREADS) k_sell_spmv_wave(SellView v, const T *x, T *y) {
+    pdl_launch_next();
+    const int u = blockIdx.x * WAVE_THREADS + threadIdx.x;
+    RowHead<T, NB> h;
+    if (u < ((v.nrows + 31) & ~31)) h.load(v, u, v.nrows);
+    pdl_wait_previous();
+    const T acc = h.sum(v, x);
+    if (h.i >= 0) y[h.i] = acc;
+}
+
+template <class T, int NB>
+__global__ void __launch_bounds__(WAVE_THREADS) k_sell_sweep_wave(SellView v, const int *copy, int ncopy, const T *b,
+                                                                  const T *x, T *xo) {
+    pdl_launch_next();
+    const int u = blockIdx.x * WAVE_THREADS + threadIdx.x, nthr = (v.nrows + 31) & ~31;
+    if (u >= nthr) {   // a warp has rows or copies, never both
+        const int j = u - nthr < ncopy ? __ldg(copy + (u - nthr)) : -1;
+        pdl_wait_previous();
+        if (j >= 0) xo[j] = x[j];
+        return;
+    }
+    RowHead<T, NB> h;
+    h.load(v, u, v.nrows);
+    const T d = h.i >= 0 ? __ldg(static_cast<const T *>(v.dinv) + u) : T(0);
+    pdl_wait_previous();
+    T bi = T(0), xi = T(0);
+    if (h.i >= 0) {
+        bi = b[h.i];
+        xi = x[h.i];
+    }
+    const T acc = h.sum(v, x);
+    if (h.i >= 0) xo[h.i] = fma(d, bi - acc, xi);
+}
+
 // One-point interpolation (one-point P, or the identity blocks of the nodal hierarchy: at most one entry per
 // row, every entry 1): x_i = x_c[col_i] + 0, or 0 for a row without an entry -- the bits of fma(1, x_c[col_i], 0)
 // that the sliced-ELL product gives (a -0 becomes +0). One column per row from the dense column array, one
@@ -364,10 +466,27 @@ __global__ void __launch_bounds__(256) k_p1_interp(int n, const int *__restrict_
     }
 }
 
+// the same in one wave, a row per thread: the column is read before the previous kernel has finished
+template <class T>
+__global__ void __launch_bounds__(256) k_p1_interp_wave(int n, const int *p1col, const int *blk_sys, const uint8_t *run,
+                                                        const T *xc, T *x) {
+    pdl_launch_next();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    bool on = i < n;
+    if (on && run) {
+        const int q = blk_sys[i >> 5];
+        on = q < 0 || run[q];
+    }
+    const int c = on ? __ldg(p1col + i) : -1;
+    pdl_wait_previous();
+    if (on) x[i] = c >= 0 ? xc[c] + T(0) : T(0);
+}
+
 template <class T>
 void p1_interp(int n, const int *p1col, const int *blk_sys, const uint8_t *run, const T *xc, T *x, cudaStream_t s) {
     if (n <= 0) return;
-    launch_pdl(k_p1_interp<T>, grid_for(n, 256, device_sms() * 16), 256, 0, s, n, p1col, blk_sys, run, xc, x);
+    if (n <= one_wave_rows<T>()) launch_pdl(k_p1_interp_wave<T>, (n + 255) / 256, 256, 0, s, n, p1col, blk_sys, run, xc, x);
+    else launch_pdl(k_p1_interp<T>, grid_for(n, 256, device_sms() * 16), 256, 0, s, n, p1col, blk_sys, run, xc, x);
     count_launch();
 }
 template void p1_interp<float>(int, const int *, const int *, const uint8_t *, const float *, float *, cudaStream_t);
@@ -375,23 +494,24 @@ template void p1_interp<double>(int, const int *, const int *, const uint8_t *, 
                                 cudaStream_t);
 
 // ---------------------------------------------------------------------------------------
-// The bottom of the V-cycle in one thread-block cluster: the restrictions of the smallest levels, the coarsest
-// solve, and on the way up their interpolations and F/C sweeps, with a cluster barrier between phases instead of a
-// kernel boundary. Every row is computed by one thread with the arithmetic of k_sell_spmv, k_sell_sweep, k_p1_interp
-// and k_dense_apply (same entries, same order), so the cycle's result is the same bits either way. Stopped batched
-// systems are not skipped here.
+// The bottom of the V-cycle in one launch: the restrictions of the smallest levels, the coarsest solve, and on the way
+// up their interpolations and F/C sweeps, in one CTA with a block barrier between phases instead of a kernel boundary.
+// Every row is computed by one thread with the arithmetic of k_sell_spmv, k_sell_sweep, k_p1_interp and k_dense_apply
+// (same entries, same order), so the cycle's result is the same bits either way. Stopped batched systems are not
+// skipped here.
 //
-// What bounds it is latency: each phase is a chain slice offset -> column -> gathered x -> fma, which costs 3-8 us a
-// phase as a kernel of its own that reads L2, however few rows there are. So everything the phases read lies in
-// shared memory: slice q of a view belongs to CTA q mod 8, whose part of all levels (row lists, diagonals, entries
-// with 16-bit columns, its rows of the coarsest inverse) lies ready in one contiguous image, packed when the
-// hierarchy is built (k_bottom_pack) and copied with 16-byte cp.async before the kernel waits for its predecessor
-// (the image does not depend on it). Each CTA also holds all vectors of all bottom levels; a row's new value is
-// written into the eight copies through distributed shared memory. Views that do not fit are read from global
-// memory eight entries at a time. Eight CTAs rather than one, because on one SM the FP64 phases and the FP64 coarsest
-// product are bound by its two FP64 lanes (a 128 x 128 product takes 10 us there) and its shared memory ends at
-// about 1,000 rows.
-// Figures: see BOTTOM_ROWS in setup_kernels.cuh.
+// What bounds it is latency: read from L2, the chain slice offset -> column -> gathered x -> fma costs over a
+// microsecond a phase however few rows there are. So everything the phases read lies in shared memory: level
+// descriptors, row lists, diagonals and as many of the views' entries as fit (with 16-bit columns) lie ready in one
+// contiguous image, packed when the hierarchy is built (k_bottom_pack), which the kernel copies with 16-byte cp.async
+// before it waits for its predecessor (the image does not depend on it). The vectors live in shared memory too. A phase
+// then takes 500 to 900 cycles in FP32. Views that do not fit are read from global memory eight entries at a time.
+//
+// The coarsest product is n^2 FP64 operations on an SM with two FP64 lanes (10 us for n = 128): the CTA is the first of
+// a cluster of BOTTOM_CTAS, whose others wait at the cluster barrier, take their share of the rows of that product and
+// write them back through distributed shared memory. Spreading the other phases over the cluster as well was slower:
+// a cluster barrier after rows were written to eight copies of x takes 1,300 to 2,800 cycles, a block barrier 80.
+// 512^2 FD one-point FP32: V-cycle 107 us with a kernel per phase down to the coarsest level, 98 us with this.
 // ---------------------------------------------------------------------------------------
 namespace {
 
@@ -400,26 +520,27 @@ __device__ __forceinline__ const T *bottom_at(const unsigned char *sm, int off) 
     return reinterpret_cast<const T *>(sm + off);
 }
 
-__device__ __forceinline__ void cluster_arrive() {
+__device__ __forceinline__ void cluster_barrier() {
     __syncwarp();   // .aligned: the warp arrives as one
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-
-// v at byte offset off of the shared memory of every CTA of the cluster (base[q]: where CTA q's begins)
-__device__ __forceinline__ void bottom_put(const unsigned (&base)[BOTTOM_CTAS], int off, float v) {
-#pragma unroll
-    for (int q = 0; q < BOTTOM_CTAS; ++q)
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(base[q] + off), "f"(v) : "memory");
-}
-__device__ __forceinline__ void bottom_put(const unsigned (&base)[BOTTOM_CTAS], int off, double v) {
-#pragma unroll
-    for (int q = 0; q < BOTTOM_CTAS; ++q)
-        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(base[q] + off), "d"(v) : "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// the sum of this thread's row of the view against x (shared), entries in ascending order as everywhere; warp w of
-// the CTA holds the CTA's w-th slice of the view
+// the value at shared-memory address a of the cluster, and a store to one
+__device__ __forceinline__ void far_load(unsigned a, float &v) {
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void far_load(unsigned a, double &v) {
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void far_store(unsigned a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void far_store(unsigned a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
+// the sum of this thread's row of the view against x (shared), entries in ascending order as everywhere
 template <class T>
 __device__ __forceinline__ T bottom_row(const unsigned char *sm, const BottomView<T> &v, const T *x) {
     const int lane = threadIdx.x & 31;
@@ -450,56 +571,45 @@ __device__ __forceinline__ T bottom_row(const unsigned char *sm, const BottomVie
     return acc;
 }
 
-// y = (view) x, y at byte offset o_y
+// y = (view) x
 template <class T>
-__device__ __forceinline__ void bottom_spmv(const unsigned char *sm, const unsigned (&base)[BOTTOM_CTAS],
-                                            const BottomView<T> &v, const T *x, int o_y) {
-    if ((int)(threadIdx.x >> 5) >= v.nloc) return;
+__device__ __forceinline__ void bottom_spmv(const unsigned char *sm, const BottomView<T> &v, const T *x, T *y) {
+    if ((int)threadIdx.x >= v.nrows) return;
     const T acc = bottom_row<T>(sm, v, x);
-    const int i = bottom_at<uint16_t>(sm, v.o_row)[threadIdx.x];
-    if (i != BOTTOM_NOROW) bottom_put(base, o_y + i * (int)sizeof(T), acc);
+    y[bottom_at<uint16_t>(sm, v.o_row)[threadIdx.x]] = acc;
 }
 
-// one Jacobi sweep in place: the new values are written once every CTA has read the old ones
+// one Jacobi sweep in place: the new values are written once all rows have read the old ones
 template <class T>
-__device__ __forceinline__ void bottom_sweep(const unsigned char *sm, const unsigned (&base)[BOTTOM_CTAS],
-                                             const BottomView<T> &v, const T *b, int o_x) {
-    const T *x = bottom_at<T>(sm, o_x);
-    int i = BOTTOM_NOROW;
+__device__ __forceinline__ void bottom_sweep(const unsigned char *sm, const BottomView<T> &v, const T *b, T *x) {
+    const bool in = (int)threadIdx.x < v.nrows;
+    int i = 0;
     T xn = T(0);
-    if ((int)(threadIdx.x >> 5) < v.nloc) {
+    if (in) {
         i = bottom_at<uint16_t>(sm, v.o_row)[threadIdx.x];
         const T acc = bottom_row<T>(sm, v, x);
-        if (i != BOTTOM_NOROW) xn = fma(bottom_at<T>(sm, v.o_dinv)[threadIdx.x], b[i] - acc, x[i]);
+        xn = fma(bottom_at<T>(sm, v.o_dinv)[threadIdx.x], b[i] - acc, x[i]);
     }
-    cluster_arrive();
-    cluster_wait();
-    if (i != BOTTOM_NOROW) bottom_put(base, o_x + i * (int)sizeof(T), xn);
-    cluster_arrive();
-    cluster_wait();
+    __syncthreads();
+    if (in) x[i] = xn;
+    __syncthreads();
 }
 
 }  // namespace
 
-// Lays the image of CTA blockIdx.y out and fills the part of view blockIdx.x (four per level: R, P, AF, AC). The
-// entries of a view go into the image as long as they fit in cap bytes, deepest level first and the F rows (swept
-// twice) before the others; every block works the layout out for itself from the slices' lengths. lv: the levels with
-// the offsets of lists and vectors already set (host). The image starts with its own size, then the descriptors;
-// entries take the bytes from o_entries up to cap. Ainv's rows go to o_ainv (when >= 0).
+// Lays the image out and fills it, one CTA per view (four per level: R, P, AF, AC). The entries of a view go into the
+// image as long as they fit in cap bytes, deepest level first and the F rows (swept twice) before the others; every CTA
+// works the layout out for itself from the views' lengths. lv: the levels with the offsets of lists and vectors already
+// set (host). The image starts with its own size, then the descriptors; entries take the bytes from o_entries on.
 template <class T>
-__global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom_pack(const BottomLevel<T> *__restrict__ lv, int nl, int o_desc,
-                                                                int o_entries, int cap, int nz,
-                                                                const double *__restrict__ Ainv, int o_ainv,
-                                                                unsigned char *__restrict__ images) {
-    __shared__ int ofs[4 * BOTTOM_LEVELS], num[4 * BOTTOM_LEVELS], total;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nv = 4 * nl, rank = blockIdx.y;
-    unsigned char *img = images + (size_t)rank * BOTTOM_SMEM;
-    for (int q = w; q < nv; q += BOTTOM_THREADS / 32) {
+__global__ void __launch_bounds__(256) k_bottom_pack(const BottomLevel<T> *__restrict__ lv, int nl, int o_desc,
+                                                     int o_entries, int cap, unsigned char *__restrict__ img) {
+    __shared__ int ofs[4 * BOTTOM_LEVELS], beg[4 * BOTTOM_LEVELS], num[4 * BOTTOM_LEVELS], total;
+    const int t = threadIdx.x, nv = 4 * nl;
+    for (int q = t; q < nv; q += blockDim.x) {
         const BottomView<T> &v = lv[q >> 2].v[q & 3];
-        const int s = lane * BOTTOM_CTAS + rank;
-        int c = 32 * s < v.nrows ? v.ptr[s + 1] - v.ptr[s] : 0;
-        c = __reduce_add_sync(0xffffffffu, c);
-        if (lane == 0) num[q] = c;
+        beg[q] = v.nrows > 0 ? v.ptr[0] : 0;
+        num[q] = v.nrows > 0 ? v.ptr[(v.nrows + 31) >> 5] - beg[q] : 0;
     }
     __syncthreads();
     if (t == 0) {
@@ -522,148 +632,143 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom_pack(const BottomLeve
     if (q == 0) {
         if (t < 4) reinterpret_cast<int *>(img)[t] = t == 0 ? total : 0;
         const int words = nl * (int)(sizeof(BottomLevel<T>) / sizeof(int));
-        for (int k = t; k < words; k += BOTTOM_THREADS)
+        for (int k = t; k < words; k += blockDim.x)
             reinterpret_cast<int *>(img + o_desc)[k] = reinterpret_cast<const int *>(lv)[k];
         __syncthreads();
-        for (int p = t; p < nv; p += BOTTOM_THREADS) {
+        for (int p = t; p < nv; p += blockDim.x) {
             BottomView<T> &v = reinterpret_cast<BottomLevel<T> *>(img + o_desc)[p >> 2].v[p & 3];
-            const int nsl = (v.nrows + 31) >> 5;
-            v.nloc = nsl > rank ? (nsl - rank + BOTTOM_CTAS - 1) / BOTTOM_CTAS : 0;
             v.o_val = ofs[p];
             v.o_col = ofs[p] >= 0 ? ofs[p] + num[p] * (int)sizeof(T) : -1;
         }
-        if (o_ainv >= 0)
-            for (int k = t; k < nz * ((nz - rank + BOTTOM_CTAS - 1) / BOTTOM_CTAS); k += BOTTOM_THREADS)
-                reinterpret_cast<double *>(img + o_ainv)[k] = Ainv[(size_t)(rank + k / nz * BOTTOM_CTAS) * nz + k % nz];
     }
     const BottomLevel<T> &L = lv[q >> 2];
     const BottomView<T> &v = L.v[q & 3];
-    if ((q & 3) == BOTTOM_P && L.p1col) {
-        const int i = (w * BOTTOM_CTAS + rank) * 32 + lane;
-        if (i < L.n) reinterpret_cast<int16_t *>(img + L.o_p1)[t] = (int16_t)L.p1col[i];
+    if ((q & 3) == BOTTOM_P && L.p1col)
+        for (int k = t; k < L.n; k += blockDim.x) reinterpret_cast<int16_t *>(img + L.o_p1)[k] = (int16_t)L.p1col[k];
+    for (int k = t; k < v.nrows; k += blockDim.x) {
+        reinterpret_cast<uint16_t *>(img + v.o_row)[k] = (uint16_t)v.row[k];
+        if (v.dinv) reinterpret_cast<T *>(img + v.o_dinv)[k] = v.dinv[k];
     }
-    // warp w: the CTA's w-th slice
-    const int s = w * BOTTOM_CTAS + rank, u = 32 * s + lane;
-    if (32 * s >= v.nrows) return;
-    reinterpret_cast<uint16_t *>(img + v.o_row)[t] = u < v.nrows ? (uint16_t)v.row[u] : (uint16_t)BOTTOM_NOROW;
-    if (v.dinv && u < v.nrows) reinterpret_cast<T *>(img + v.o_dinv)[t] = v.dinv[u];
-    const int beg = v.ptr[s], len = (v.ptr[s + 1] - beg) >> 5;
-    int loc = 0;   // entries of the CTA's slices before this one
-    for (int k = lane; k < w; k += 32) loc += v.ptr[k * BOTTOM_CTAS + rank + 1] - v.ptr[k * BOTTOM_CTAS + rank];
-    loc = __reduce_add_sync(0xffffffffu, loc);
-    if (lane == 0) reinterpret_cast<int2 *>(img + v.o_ptr)[w] = make_int2(ofs[q] >= 0 ? loc : beg, len);
+    for (int k = t; k < (v.nrows + 31) >> 5; k += blockDim.x) {
+        const int a = v.ptr[k];
+        reinterpret_cast<int2 *>(img + v.o_ptr)[k] = make_int2(ofs[q] >= 0 ? a - beg[q] : a, (v.ptr[k + 1] - a) >> 5);
+    }
     if (ofs[q] < 0) return;
-    T *val = reinterpret_cast<T *>(img + ofs[q]) + loc + lane;
-    uint16_t *col = reinterpret_cast<uint16_t *>(img + ofs[q] + num[q] * (int)sizeof(T)) + loc + lane;
+    T *val = reinterpret_cast<T *>(img + ofs[q]);
+    uint16_t *col = reinterpret_cast<uint16_t *>(img + ofs[q] + num[q] * (int)sizeof(T));
 #pragma unroll 4
-    for (int j = 0; j < len; ++j) {
-        val[32 * j] = v.val[beg + lane + 32 * j];
-        col[32 * j] = (uint16_t)v.col[beg + lane + 32 * j];
+    for (int k = t; k < num[q]; k += blockDim.x) {
+        val[k] = v.val[beg[q] + k];
+        col[k] = (uint16_t)v.col[beg[q] + k];
     }
 }
 
 template <class T>
 __global__ void __cluster_dims__(BOTTOM_CTAS, 1, 1) __launch_bounds__(BOTTOM_THREADS) k_cycle_bottom(BottomArgs<T> a) {
     extern __shared__ __align__(16) unsigned char sm[];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5, rank = blockIdx.x;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, rank = blockIdx.x, n = a.nc, nl = a.nl;
+    const int mine = n > rank ? (n - rank + BOTTOM_CTAS - 1) / BOTTOM_CTAS : 0;   // rows rank, rank + 8, ... of Ainv
+    pdl_launch_next();
     const unsigned own = (unsigned)__cvta_generic_to_shared(sm);
-    {
-        const unsigned char *img = a.img + (size_t)rank * BOTTOM_SMEM;
-        const int total = __ldg(reinterpret_cast<const int *>(img));
+    unsigned first;   // the first CTA's shared memory
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(first) : "r"(own));
+    if (rank == 0) {
+        const int total = __ldg(reinterpret_cast<const int *>(a.img));
         for (int k = 16 * t; k < total; k += 16 * BOTTOM_THREADS)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(own + k), "l"(img + k) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(own + k), "l"(a.img + k) : "memory");
     }
-    unsigned base[BOTTOM_CTAS];
-#pragma unroll
-    for (int q = 0; q < BOTTOM_CTAS; ++q)
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base[q]) : "r"(own), "r"(q));
+    if (a.o_ainv >= 0)
+        for (int k = t; k < mine * n; k += BOTTOM_THREADS)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(own + a.o_ainv + 8 * k),
+                         "l"(a.Ainv + (size_t)(rank + k / n * BOTTOM_CTAS) * n + k % n)
+                         : "memory");
     asm volatile("cp.async.wait_all;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int k = t; k < a.n0; k += BOTTOM_THREADS) reinterpret_cast<T *>(sm + a.o_b0)[k] = a.b[k];
-    cluster_arrive();   // every CTA runs and holds its image
-    cluster_wait();
-    const int nl = a.nl;
-    const BottomLevel<T> *lv = bottom_at<BottomLevel<T>>(sm, a.o_desc);
-    for (int l = 0; l < nl; ++l) {
-        bottom_spmv<T>(sm, base, lv[l].v[BOTTOM_R], bottom_at<T>(sm, lv[l].o_b), l + 1 < nl ? lv[l + 1].o_b : a.o_cb);
-        cluster_arrive();
-        cluster_wait();
-    }
-    {
-        // x = Ainv b, row rank + 8 k in this CTA, four rows per warp. A lane sums its columns in ascending order and
-        // the lanes' sums are added in k_dense_apply's butterfly order (16, 8, 4, 2, 1), but four rows share the first
-        // two steps: each half, then each quarter of the warp goes on with its own rows (a warp FP64 instruction
-        // costs 16 cycles of the SM whatever its lanes hold).
-        const int n = a.nc, mine = n > rank ? (n - rank + BOTTOM_CTAS - 1) / BOTTOM_CTAS : 0;
-        const T *cb = bottom_at<T>(sm, a.o_cb);
-        for (int r0 = 4 * w; r0 < mine; r0 += 4 * (BOTTOM_THREADS / 32)) {
-            double acc[4] = {0.0, 0.0, 0.0, 0.0};
-            if (a.o_ainv >= 0) {
-                const double *A = bottom_at<double>(sm, a.o_ainv) + r0 * n;
-#pragma unroll 2
-                for (int c = lane; c < n; c += 32) {
-                    const double xc = (double)cb[c];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (r0 + k < mine) acc[k] = fma(A[k * n + c], xc, acc[k]);
-                }
-            } else {
-                const double *A = a.Ainv + (size_t)(rank + r0 * BOTTOM_CTAS) * n;
-#pragma unroll 4
-                for (int c = lane; c < n; c += 32) {
-                    const double xc = (double)cb[c];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (r0 + k < mine) acc[k] = fma(__ldg(A + (size_t)k * BOTTOM_CTAS * n + c), xc, acc[k]);
-                }
-            }
-            const bool h16 = lane & 16, h8 = lane & 8;
-            const double s0 = __shfl_xor_sync(0xffffffffu, h16 ? acc[0] : acc[2], 16);
-            const double s1 = __shfl_xor_sync(0xffffffffu, h16 ? acc[1] : acc[3], 16);
-            const double p0 = (h16 ? acc[2] : acc[0]) + s0, p1 = (h16 ? acc[3] : acc[1]) + s1;
-            double v = (h8 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h8 ? p0 : p1, 8);
-            for (int o = 4; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            const int k = (h16 ? 2 : 0) + (h8 ? 1 : 0);
-            if ((lane & 7) == 0 && r0 + k < mine)
-                bottom_put(base, a.o_cx + (rank + (r0 + k) * BOTTOM_CTAS) * (int)sizeof(T), (T)v);
+    const BottomLevel<T> *lv = bottom_at<BottomLevel<T>>(sm, a.o_desc);   // rank 0 only
+    T *cb = reinterpret_cast<T *>(sm + a.o_cb);
+    if (rank == 0) {
+        pdl_wait_previous();
+        if (t < a.n0) reinterpret_cast<T *>(sm + a.o_b0)[t] = a.b[t];
+        __syncthreads();
+        for (int l = 0; l < nl; ++l) {
+            bottom_spmv<T>(sm, lv[l].v[BOTTOM_R], bottom_at<T>(sm, lv[l].o_b),
+                           l + 1 < nl ? reinterpret_cast<T *>(sm + lv[l + 1].o_b) : cb);
+            __syncthreads();
         }
-        cluster_arrive();
-        cluster_wait();
     }
+    cluster_barrier();   // the coarsest right-hand side is complete in the first CTA
+    if (rank > 0) {
+        if (t < n) {
+            T v;
+            far_load(first + a.o_cb + t * (int)sizeof(T), v);
+            cb[t] = v;
+        }
+        __syncthreads();
+    }
+    // x = Ainv b, row rank + 8 k in this CTA, four rows per warp. A lane sums its columns in ascending order and the
+    // lanes' sums are added in k_dense_apply's butterfly order (16, 8, 4, 2, 1), but four rows share the first two
+    // steps: each half, then each quarter of the warp goes on with its own rows (a warp FP64 instruction takes 19
+    // cycles of the SM whatever its lanes hold).
+    for (int r0 = 4 * w; r0 < mine; r0 += 4 * (BOTTOM_THREADS / 32)) {
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        if (a.o_ainv >= 0) {
+            const double *A = bottom_at<double>(sm, a.o_ainv) + r0 * n;
+#pragma unroll 2
+            for (int c = lane; c < n; c += 32) {
+                const double xc = (double)cb[c];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (r0 + k < mine) acc[k] = fma(A[k * n + c], xc, acc[k]);
+            }
+        } else {
+            const double *A = a.Ainv + (size_t)(rank + r0 * BOTTOM_CTAS) * n;
+#pragma unroll 4
+            for (int c = lane; c < n; c += 32) {
+                const double xc = (double)cb[c];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (r0 + k < mine) acc[k] = fma(__ldg(A + (size_t)k * BOTTOM_CTAS * n + c), xc, acc[k]);
+            }
+        }
+        const bool h16 = lane & 16, h8 = lane & 8;
+        const double s0 = __shfl_xor_sync(0xffffffffu, h16 ? acc[0] : acc[2], 16);
+        const double s1 = __shfl_xor_sync(0xffffffffu, h16 ? acc[1] : acc[3], 16);
+        const double p0 = (h16 ? acc[2] : acc[0]) + s0, p1 = (h16 ? acc[3] : acc[1]) + s1;
+        double v = (h8 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h8 ? p0 : p1, 8);
+        for (int o = 4; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        const int k = (h16 ? 2 : 0) + (h8 ? 1 : 0);
+        if ((lane & 7) == 0 && r0 + k < mine)
+            far_store(first + a.o_cx + (rank + (r0 + k) * BOTTOM_CTAS) * (int)sizeof(T), (T)v);
+    }
+    cluster_barrier();   // the coarsest solution is complete in the first CTA
+    if (rank > 0) return;
     const int sq[3] = {a.seq.x, a.seq.y, a.seq.z};
     for (int l = nl - 1; l >= 0; --l) {
         const BottomLevel<T> &L = lv[l];
         const T *xc = bottom_at<T>(sm, l + 1 < nl ? lv[l + 1].o_x : a.o_cx);
+        T *x = reinterpret_cast<T *>(sm + L.o_x);
         if (L.p1col) {
-            const int i = (w * BOTTOM_CTAS + rank) * 32 + lane;
-            if (i < L.n) {
+            if (t < L.n) {
                 const int c = bottom_at<int16_t>(sm, L.o_p1)[t];
-                bottom_put(base, L.o_x + i * (int)sizeof(T), c >= 0 ? xc[c] + T(0) : T(0));
+                x[t] = c >= 0 ? xc[c] + T(0) : T(0);
             }
         } else {
-            bottom_spmv<T>(sm, base, L.v[BOTTOM_P], xc, L.o_x);
+            bottom_spmv<T>(sm, L.v[BOTTOM_P], xc, x);
         }
-        cluster_arrive();
-        cluster_wait();
+        __syncthreads();
         for (int k = 0; k < 3 && sq[k] >= 0; ++k)
-            bottom_sweep<T>(sm, base, L.v[sq[k] == CF_F ? BOTTOM_AF : BOTTOM_AC], bottom_at<T>(sm, L.o_b), L.o_x);
+            bottom_sweep<T>(sm, L.v[sq[k] == CF_F ? BOTTOM_AF : BOTTOM_AC], bottom_at<T>(sm, L.o_b), x);
     }
-    for (int k = rank * BOTTOM_THREADS + t; k < a.n0; k += BOTTOM_CTAS * BOTTOM_THREADS)
-        a.x[k] = reinterpret_cast<const T *>(sm + a.o_x0)[k];
+    if (t < a.n0) a.x[t] = bottom_at<T>(sm, a.o_x0)[t];
 }
 
 template <class T>
-void bottom_pack(const BottomLevel<T> *lv, int nl, int o_desc, int o_entries, int cap, int nz, const double *Ainv,
-                 int o_ainv, unsigned char *images, cudaStream_t s) {
-    k_bottom_pack<T><<<dim3(4 * nl, BOTTOM_CTAS), BOTTOM_THREADS, 0, s>>>(lv, nl, o_desc, o_entries, cap, nz, Ainv, o_ainv,
-                                                                          images);
+void bottom_pack(const BottomLevel<T> *lv, int nl, int o_desc, int o_entries, int cap, unsigned char *img,
+                 cudaStream_t s) {
+    k_bottom_pack<T><<<4 * nl, 256, 0, s>>>(lv, nl, o_desc, o_entries, cap, img);
     count_launch();
 }
-template void bottom_pack<float>(const BottomLevel<float> *, int, int, int, int, int, const double *, int, unsigned char *,
-                                 cudaStream_t);
-template void bottom_pack<double>(const BottomLevel<double> *, int, int, int, int, int, const double *, int,
-                                  unsigned char *, cudaStream_t);
+template void bottom_pack<float>(const BottomLevel<float> *, int, int, int, int, unsigned char *, cudaStream_t);
+template void bottom_pack<double>(const BottomLevel<double> *, int, int, int, int, unsigned char *, cudaStream_t);
 
 // whether the device can hold the bottom kernel's cluster
 template <class T>
@@ -792,6 +897,13 @@ void launch_sell_fill_multi(const SellDesc *d, int p0, int p1, int lin_beg, int 
 template <class T>
 void sell_spmv(const SellView &v, const T *x, T *y, cudaStream_t s) {
     if (v.nrows <= 0) return;
+    if (v.tb == 0 && v.nrows <= one_wave_rows<T>()) {
+        const int grid = (v.nrows + WAVE_THREADS - 1) / WAVE_THREADS;
+        if (v.long_rows) launch_pdl(k_sell_spmv_wave<T, 16>, grid, WAVE_THREADS, 0, s, v, x, y);
+        else launch_pdl(k_sell_spmv_wave<T, 8>, grid, WAVE_THREADS, 0, s, v, x, y);
+        count_launch();
+        return;
+    }
     // every row is summed alone by one thread, so the schedule (block size, grid cap, rows per thread) never
     // changes the result
     const int tb = v.tb > 0 ? v.tb : 256;
@@ -805,6 +917,13 @@ void sell_spmv(const SellView &v, const T *x, T *y, cudaStream_t s) {
 template <class T>
 void sell_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const T *x, T *xo, cudaStream_t s) {
     if (v.nrows + ncopy <= 0) return;
+    if (v.tb == 0 && v.nrows + ncopy <= one_wave_rows<T>()) {
+        const int grid = (((v.nrows + 31) & ~31) + ncopy + WAVE_THREADS - 1) / WAVE_THREADS;
+        if (v.long_rows) launch_pdl(k_sell_sweep_wave<T, 16>, grid, WAVE_THREADS, 0, s, v, copy, ncopy, b, x, xo);
+        else launch_pdl(k_sell_sweep_wave<T, 8>, grid, WAVE_THREADS, 0, s, v, copy, ncopy, b, x, xo);
+        count_launch();
+        return;
+    }
     const int tb = v.tb > 0 ? v.tb : 256;
     const int cap = v.grid > 0 ? v.grid : device_sms() * 16;
     const long long nsl = (v.nrows + 31) / 32;

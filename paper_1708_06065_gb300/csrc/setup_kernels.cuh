@@ -14,6 +14,7 @@ struct SellView {
     int *row = nullptr;         // view row -> matrix row
     void *dinv = nullptr;       // Jacobi diagonal per view row (sweep views), same type as val
     int tb = 0, grid = 0;       // launch schedule picked by the autotuner (0: 256 threads, grid capped at 16 blocks per SM)
+    bool long_rows = false;     // more than WAVE_SHORT entries a row on average (the one-wave kernels' variants)
     int rpt = 1;                // rows per thread (1 or 2: rows of two consecutive slices, same lane)
     // batched systems: the system of every slice (-1: rows of several systems) and the per-system run flags;
     // slices of a stopped system are skipped (their outputs keep older values). NULL: every slice runs.
@@ -21,6 +22,14 @@ struct SellView {
     const uint8_t *run = nullptr;
     bool zero_stopped = false;  // products: write 0 to the rows of a stopped system's slices instead of skipping them
 };
+
+// One-wave kernels (sell.cu): views of at most WAVE_BYTES_PER_SM / sizeof(T) rows per SM (2,048 in FP32, a full SM of
+// threads; 1,024 in FP64, whose registers allow half of that); rows of more than WAVE_SHORT entries on average read 16
+// entries ahead instead of 8. V-cycle with 0 / 512 / 1,024 / 2,048 / 4,096 FP32 rows per SM: 512^2 FD 152 / 134 / 128 /
+// 121 / 120 us, 128^3 314 / 304 / 292 / 281 / 279 us; FP64 0 / 512 / 1,024 / 2,048: 101^3 299 / 273 / 259 / 253 us,
+// 24 systems 253 / 222 / 217 / 223 us.
+constexpr int WAVE_SHORT = 6;
+constexpr int WAVE_BYTES_PER_SM = 8192;
 
 // ---- setup_graph.cu -------------------------------------------------------------------
 constexpr int SMALL_SCAN_MAX = 65536;   // exclusive scans up to this length run in one CTA
@@ -222,6 +231,8 @@ struct SellDesc {
 void launch_sell_prepare_multi(const SellDesc *d, int nd, int nwin, int nlin, int *cnt, unsigned long long *gsum,
                                cudaStream_t s);
 void launch_sell_fill_multi(const SellDesc *d, int p0, int p1, int lin_beg, int lin_end, bool fp32, cudaStream_t s);
+// the largest view that the one-wave kernels take
+template <class T> long long one_wave_rows() { return (long long)device_sms() * (WAVE_BYTES_PER_SM / (int)sizeof(T)); }
 template <class T> void sell_spmv(const SellView &v, const T *x, T *y, cudaStream_t s);
 template <class T>
 void sell_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const T *x, T *xo, cudaStream_t s);
@@ -231,15 +242,14 @@ void sell_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const
 // blocks of stopped systems are skipped
 template <class T>
 void p1_interp(int n, const int *p1col, const int *blk_sys, const uint8_t *run, const T *xc, T *x, cudaStream_t s);
-// the bottom of the V-cycle in one cluster of BOTTOM_CTAS CTAs (sell.cu): levels of at most BOTTOM_ROWS rows, at most
-// one row of a view per thread. A level: R restricts b to the next level, P interpolates (sliced ELL, or the one-point
-// column array p1col when set), AF / AC sweep the F / C rows; the coarsest: x = Ainv b. o_*: byte offsets in a CTA's
-// shared memory, which begins with the CTA's packed image of what the phases read (bottom_pack) and ends with the
-// levels' vectors. nloc: the CTA's slices of the view; o_val < 0: the entries did not fit and are read from col / val.
+// the bottom of the V-cycle in one launch (sell.cu): levels of at most BOTTOM_ROWS rows, one row of a view per thread of
+// the first CTA. A level: R restricts b to the next level, P interpolates (sliced ELL, or the one-point column array
+// p1col when set), AF / AC sweep the F / C rows; the coarsest: x = Ainv b over the cluster. o_*: byte offsets in shared
+// memory, which begins with the packed image of what the phases read (bottom_pack) and ends with the levels' vectors;
+// o_val < 0: the entries did not fit and are read from col / val.
 constexpr int BOTTOM_R = 0, BOTTOM_P = 1, BOTTOM_AF = 2, BOTTOM_AC = 3;
-constexpr int BOTTOM_NOROW = 0xffff;
 template <class T> struct BottomView {
-    int nrows = 0, nloc = 0, o_ptr = 0, o_row = 0, o_dinv = 0, o_val = -1, o_col = -1, pad = 0;
+    int nrows = 0, o_ptr = 0, o_row = 0, o_dinv = 0, o_val = -1, o_col = -1;
     const int *ptr = nullptr, *row = nullptr, *col = nullptr;
     const T *val = nullptr, *dinv = nullptr;
 };
@@ -249,7 +259,7 @@ template <class T> struct BottomLevel {
     BottomView<T> v[4];
 };
 template <class T> struct BottomArgs {
-    const unsigned char *img = nullptr;          // BOTTOM_CTAS images, BOTTOM_SMEM bytes apart
+    const unsigned char *img = nullptr;
     int nl = 0, n0 = 0, nc = 0;                  // bottom levels above the coarsest, rows of the first, of the coarsest
     int o_desc = 0, o_b0 = 0, o_x0 = 0, o_cb = 0, o_cx = 0, o_ainv = -1;
     const double *Ainv = nullptr;
@@ -257,17 +267,21 @@ template <class T> struct BottomArgs {
     T *x = nullptr;
     int4 seq = {-1, -1, -1, 0};                  // the sweep targets (CF_F / CF_C, -1 ends)
 };
-// Whole V-cycle, one CTA reading L2 up to 1,024 rows -> one cluster up to 8,192 rows: 512^2 FD, FP32 one-point
-// 176 -> 151 us; 301^2 FD, FP64 lAIP 302 -> 228 us; 64^2 FD, FP64 lAIP 114 -> 95 us. A phase takes 0.7 us (a product) to
-// 1.1 us (a sweep), against 2.5 to 6 us as a kernel in the captured graph; 8,192 is one row per thread of the cluster.
 constexpr int BOTTOM_CTAS = 8;
 constexpr int BOTTOM_THREADS = 1024;
-constexpr int BOTTOM_ROWS = BOTTOM_CTAS * BOTTOM_THREADS;
+constexpr int BOTTOM_ROWS = BOTTOM_THREADS;
+// Entries of A that a level of the bottom may have: with more, one SM's shared memory (FP32) or its two FP64 lanes cost
+// more than the kernel boundaries that the bottom saves. V-cycle with limits of 1,000 / 4,096 / 8,192 / 20,000 entries
+// in FP64: 301^2 FD lAIP 174 / 174 / 165 / 170 us, 64^2 87 / 85 / 81 / 81 us; in FP32 2,000 / 5,000 / 12,288 / 20,000:
+// 512^2 FD one-point 101 / 96 / 98 / 97 us; without a bottom 177, 88 and 107 us.
+template <class T> constexpr int bottom_entries() { return sizeof(T) == 4 ? 12288 : 8192; }
 constexpr int BOTTOM_LEVELS = 25;                // more levels than this are not taken into the bottom
-constexpr int BOTTOM_SMEM = 224 * 1024;
+// Half of an SM's on-chip memory: with 224 KB the SMs that ran the bottom were left without an L1 for the streaming
+// kernels after it (192^3 V-cycle 655 -> 750 us).
+constexpr int BOTTOM_SMEM = 112 * 1024;
 template <class T>
-void bottom_pack(const BottomLevel<T> *lv, int nl, int o_desc, int o_entries, int cap, int nz, const double *Ainv,
-                 int o_ainv, unsigned char *images, cudaStream_t s);
+void bottom_pack(const BottomLevel<T> *lv, int nl, int o_desc, int o_entries, int cap, unsigned char *img,
+                 cudaStream_t s);
 template <class T> bool bottom_fits();           // also allows the kernel its shared memory: before cycle_bottom
 template <class T> void cycle_bottom(const BottomArgs<T> &a, cudaStream_t s);
 // the system of every 32-row block of a level (seg: first row of every system, nseg + 1 entries)

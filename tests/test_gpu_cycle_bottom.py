@@ -1,7 +1,7 @@
-"""The small levels of the V-cycle run in one thread-block cluster (rows and matrix entries in shared memory, the
-coarsest product spread over the cluster). Sizes around its limits: 8,192 rows in the first level, 512 unknowns in the
-coarsest, slices that do not divide among the CTAs, one bottom level, views that do not fit in shared memory (lAIP in
-FP64), every sweep order; after a refresh, and for a batch."""
+"""The V-cycle's kernels for levels that fit on the GPU at once. The smallest levels run in one CTA (matrix entries and
+vectors in shared memory, the coarsest product over a cluster), the others with one row per thread: sizes around the
+limits (1,024 rows in the first bottom level, 512 unknowns in the coarsest, entries that do not fit in shared memory,
+rows longer than the entries read ahead), every sweep order; after a refresh, and for a batch."""
 import numpy as np
 import pytest
 
@@ -25,7 +25,7 @@ def lair():
 P1 = dict(cf_mode=1, interp=1, lump_tol=0.05)
 CASES = [
     (24, dict(coarse_max=1)), (24, dict(P1, coarse_max=300)), (33, dict(coarse_max=512)), (45, dict(coarse_max=513)),
-    (90, dict()), (91, dict(P1)), (128, dict(P1)), (130, dict()), (150, dict(P1, coarse_max=8)),
+    (45, dict(P1)), (46, dict(P1)), (58, dict()), (90, dict()), (130, dict()), (150, dict(P1, coarse_max=8)),
     (181, dict(distance=2, lump_tol=0.0)), (64, dict(cf_mode=0, relax=1)), (64, dict(cf_mode=0, relax=2)),
     (100, dict(P1, relax=1)), (100, dict(P1, relax=2)),
 ]
