@@ -2121,9 +2121,10 @@ lair_status lair_precond_apply(lair_handle *h, const double *b, double *x) {
     const int n = h->H.lev[0].A.nr;
     TRY(ensure_work(h, n, 0));
     const bool bdev = is_device_ptr(b), xdev = is_device_ptr(x);
-    CU(cudaMemcpyAsync(h->wb, b, sizeof(double) * n, bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->s));
-    TRY(precond(h, h->H, h->wb, h->wx));
-    CU(cudaMemcpyAsync(x, h->wx, sizeof(double) * n, xdev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->s));
+    // device vectors are read and written where they are: b is read whole before x is written, so they may overlap
+    if (!bdev) CU(cudaMemcpyAsync(h->wb, b, sizeof(double) * n, cudaMemcpyHostToDevice, h->s));
+    TRY(precond(h, h->H, bdev ? b : h->wb, xdev ? x : h->wx));
+    if (!xdev) CU(cudaMemcpyAsync(x, h->wx, sizeof(double) * n, cudaMemcpyDeviceToHost, h->s));
     CU(cudaStreamSynchronize(h->s));
     return LAIR_OK;
 }

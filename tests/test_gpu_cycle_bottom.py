@@ -63,3 +63,18 @@ def test_batched_cycle_with_small_levels(lair, sides):
     assert st == 0 and rel.max() <= 1e-10
     import scipy.sparse.linalg as sl
     assert entrywise_rel(x.cpu().numpy(), sl.spsolve(s.to_scipy().tocsc(), s.b)) <= 1e-6
+
+
+def test_precond_on_overlapping_vectors(lair):
+    """x = M^-1 b written over b, and over a vector that shares half of it: the same as into a vector of its own."""
+    import torch
+    s = W.fd_adr_2d(70, 0.6, 1e-3, 0.1)
+    for precision in (0, 1):
+        G = lair.Hierarchy.from_system(s, device=True, precision=precision, **P1)
+        v = torch.from_numpy(np.random.default_rng(2).uniform(-1, 1, s.n)).cuda()
+        z = G.precond(v)
+        own = v.clone()
+        assert torch.equal(G.precond(own, own), z)
+        buf = torch.zeros(s.n + s.n // 2, dtype=torch.float64, device="cuda")
+        buf[:s.n] = v
+        assert torch.equal(G.precond(buf[:s.n], buf[s.n // 2:]), z)
