@@ -2229,7 +2229,6 @@ void lair_free(lair_handle *h) {
         delete h->HT;
     }
     for (void *p : h->allocs) cudaFreeAsync(p, h->s);
-    if (h->scan_tmp) cudaFreeAsync(h->scan_tmp, h->s);
     cudaStreamSynchronize(h->s);
     for (auto &p : h->pending) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
     for (auto &p : h->graph_events) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }

@@ -413,8 +413,10 @@ static inline lair_status scan(lair_handle *h, const int *cnt, int *out, int n, 
     }
     const size_t need = scan_state_bytes((long long)n + 1);
     if (need > h->scan_tmp_bytes) {
-        if (h->scan_tmp) CU(cudaFreeAsync(h->scan_tmp, h->s));
-        CU(cudaMallocAsync(&h->scan_tmp, need, h->s));
+        // from the handle's own memory: the device's default pool gives freed memory back at every synchronisation
+        char *p;
+        TRY(dalloc(h, &p, need));
+        h->scan_tmp = p;
         h->scan_tmp_bytes = need;
     }
     CU(launch_scan((long long)n + 1, cnt, out, h->scan_tmp, h->status, h->s));

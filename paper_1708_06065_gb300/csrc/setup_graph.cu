@@ -1124,59 +1124,45 @@ __global__ void k_nb_compact(int nc, const int *__restrict__ off, const int *__r
 }
 
 // -------------------------------------------------------------------------------------
-// exclusive scan of m <= SMALL_SCAN_MAX ints in one CTA, in tiles of 16384: warp w scans the
-// 512 entries [512 w, 512 w + 512) of a tile as 16 coalesced strips of 32 held in registers
+// exclusive scan of m <= SMALL_SCAN_MAX ints in one CTA of 1024 threads: warp w scans the 32 STRIPS entries from
+// 32 STRIPS w on as coalesced strips of 32 held in registers. Bound by its chain of latencies (load, shuffles, two
+// block barriers), so the number of strips follows m: with 16 strips whatever m, a set-up's scans of a few hundred
+// entries took 4.4 us each, most of it shuffles on strips past the end; beyond 16 strips the scan over many CTAs is
+// faster (40,000 entries: 14 us in three rounds of one CTA, 4.7 us by look-back).
 // -------------------------------------------------------------------------------------
-constexpr int SCAN_STRIPS = 16;
-constexpr int SCAN_TILE = 1024 * SCAN_STRIPS;
-
+template <int STRIPS>
 __global__ void __launch_bounds__(1024) k_small_scan(int m, const int *__restrict__ in, int *__restrict__ out) {
     __shared__ int wsum[32];
-    __shared__ int tile_total;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    int carry = 0;
-    for (int base = 0; base < m; base += SCAN_TILE) {
-        const int seg = base + w * 32 * SCAN_STRIPS + lane;
-        int v[SCAN_STRIPS];
+    const int seg = w * 32 * STRIPS + lane;
+    int v[STRIPS];
 #pragma unroll
-        for (int k = 0; k < SCAN_STRIPS; ++k) v[k] = seg + 32 * k < m ? in[seg + 32 * k] : 0;
-        int run = 0;
+    for (int k = 0; k < STRIPS; ++k) v[k] = seg + 32 * k < m ? in[seg + 32 * k] : 0;
+    int run = 0;
 #pragma unroll
-        for (int k = 0; k < SCAN_STRIPS; ++k) {
-            int x = v[k];
+    for (int k = 0; k < STRIPS; ++k) {
+        int x = v[k];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            v[k] = run + x - v[k];
-            run += __shfl_sync(0xffffffffu, x, 31);
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
         }
-        if (lane == 0) wsum[w] = run;
-        __syncthreads();
-        if (w == 0) {
-            const int sv = wsum[lane];
-            int x = sv;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            wsum[lane] = x - sv;
-            if (lane == 31) tile_total = x;
-        }
-        __syncthreads();
-        const int off = carry + wsum[w];
-#pragma unroll
-        for (int k = 0; k < SCAN_STRIPS; ++k)
-            if (seg + 32 * k < m) out[seg + 32 * k] = off + v[k];
-        carry += tile_total;
-        __syncthreads();
+        v[k] = run + x - v[k];
+        run += __shfl_sync(0xffffffffu, x, 31);
     }
+    if (lane == 0) wsum[w] = run;
+    __syncthreads();
+    // every warp adds up the warps before it
+    const int off = (int)__reduce_add_sync(0xffffffffu, lane < w ? (unsigned)wsum[lane] : 0u);
+#pragma unroll
+    for (int k = 0; k < STRIPS; ++k)
+        if (seg + 32 * k < m) out[seg + 32 * k] = off + v[k];
 }
 
 void small_scan(int m, const int *in, int *out, cudaStream_t s) {
-    k_small_scan<<<1, 1024, 0, s>>>(m, in, out);
+    if (m <= 1024) k_small_scan<1><<<1, 1024, 0, s>>>(m, in, out);
+    else if (m <= 4096) k_small_scan<4><<<1, 1024, 0, s>>>(m, in, out);
+    else k_small_scan<16><<<1, 1024, 0, s>>>(m, in, out);
     count_launch();
 }
 

@@ -32,7 +32,7 @@ constexpr int WAVE_SHORT = 6;
 constexpr int WAVE_BYTES_PER_SM = 8192;
 
 // ---- setup_graph.cu -------------------------------------------------------------------
-constexpr int SMALL_SCAN_MAX = 65536;   // exclusive scans up to this length run in one CTA
+constexpr int SMALL_SCAN_MAX = 16384;   // exclusive scans up to this length run in one CTA
 // exclusive scan of m ints in one pass over many CTAs (decoupled look-back); state: scan_state_bytes(m) bytes
 size_t scan_state_bytes(long long m);
 cudaError_t launch_scan(long long m, const int *in, int *out, void *state, int *status, cudaStream_t s);

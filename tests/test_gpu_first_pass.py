@@ -66,3 +66,16 @@ def test_first_pass_matches_oracle(lair, name, rs_block):
     assert [i["n"] for i in G.info()] == [L.n for L in H.levels]
     for l in range(len(H.levels) - 1):
         assert np.array_equal(G.export_cf(l)[0], H.levels[l].cf), l
+
+
+@pytest.mark.parametrize("n", [1022, 1023, 1024, 4095, 4096, 16382, 16383, 16384, 70000])
+def test_scan_lengths(lair, n):
+    """Level sizes at which the exclusive scans change from one kernel to the next."""
+    s = W.upwind_chain(n)
+    kw = dict(cf_mode=1, interp=1, strength_abs=1)
+    G = lair.Hierarchy.from_system(s, device=True, **kw)
+    H = O.Hierarchy(s, **kw)
+    assert [i["n"] for i in G.info()] == [L.n for L in H.levels]
+    for l in range(len(H.levels) - 1):
+        assert np.array_equal(G.export_csr(l, 1)[0], H.levels[l].R[0]), l
+        assert np.array_equal(G.export_csr(l + 1, 0)[0], H.levels[l + 1].A[0]), l
