@@ -1010,108 +1010,141 @@ __global__ void k_dense_inverse(int n, const double *__restrict__ LU, const int 
     }
 }
 
-// small coarsest levels (n <= DENSE_SMEM_N): the LU factorisation entirely in shared memory, one CTA, written
-// out with its row permutation for k_dense_inv_cols
+// Small coarsest levels (n <= DENSE_SMEM_N): the LU factorisation entirely in shared memory, one CTA, written
+// out with its row permutation for k_dense_inv_cols. Bound by the FP64 units: a warp FP64 instruction occupies an SM
+// for 19 cycles whatever its lanes hold and a dependent one waits 65 cycles. So
+//  * the pivot search compares the bits of |a| as integers (the order of non-negative doubles; a NaN, which no
+//    comparison of doubles would take, counts as largest, so a matrix with one still ends in NaN) inside one warp,
+//    each lane holding its rows' keys, and only that warp and one barrier stand between two columns;
+//  * a row whose multiplier is 0 is left alone: fma(-0, u, a) = a, and the elimination of a coarse operator keeps most
+//    multipliers 0 for many columns;
+//  * a warp updates whole rows, so the multiplier is loaded once and the pivot row is read without conflicts.
+// LU and inverse together: 128 unknowns (64^2 FD lAIP) 856 -> 485 us, 98 unknowns (512^2 FD one-point) 571 -> 254 us.
 constexpr int DENSE_SMEM_N = 160;   // n^2 doubles + n ints: 205 KB of the 227 KB a CTA may have
+constexpr int DENSE_WARPS = 16;
 
-__global__ void __launch_bounds__(256) k_dense_small(int n, const int *__restrict__ rp, const int *__restrict__ col,
-                                                      const double *__restrict__ val, double *__restrict__ LU,
-                                                      int *__restrict__ perm_out, int *status) {
+__global__ void __launch_bounds__(32 * DENSE_WARPS) k_dense_small(int n, const int *__restrict__ rp,
+                                                                  const int *__restrict__ col,
+                                                                  const double *__restrict__ val, double *__restrict__ LU,
+                                                                  int *__restrict__ perm_out, int *status) {
     extern __shared__ __align__(16) unsigned char smem[];
     double *D = reinterpret_cast<double *>(smem);  // n x n
     int *perm = reinterpret_cast<int *>(D + (size_t)n * n);
-    __shared__ double bv[32];
-    __shared__ int bi[32];
-    __shared__ int bad;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) D[e] = 0.0;
-    if (threadIdx.x == 0) bad = 0;
+    __shared__ int s_piv;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, T = blockDim.x, nw = T >> 5;
+    for (int e = t; e < n * n; e += T) D[e] = 0.0;
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = t; i < n; i += T) {
         perm[i] = i;
         for (int k = rp[i]; k < rp[i + 1]; ++k) D[i * n + col[k]] = val[k];
     }
     __syncthreads();
     for (int k = 0; k < n; ++k) {
-        double best = -1.0;
-        int piv = -1;
-        for (int r = k + threadIdx.x; r < n; r += blockDim.x) {
-            double v = fabs(D[r * n + k]);
-            if (piv < 0 || v > best) { best = v; piv = r; }
-        }
-        for (int o = 16; o >= 1; o >>= 1) {
-            double ov = __shfl_xor_sync(0xffffffffu, best, o);
-            int oi = __shfl_xor_sync(0xffffffffu, piv, o);
-            if (oi >= 0 && (piv < 0 || ov > best || (ov == best && oi < piv))) { best = ov; piv = oi; }
-        }
-        if ((threadIdx.x & 31) == 0) { bv[threadIdx.x >> 5] = best; bi[threadIdx.x >> 5] = piv; }
-        __syncthreads();
-        best = bv[0];
-        piv = bi[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-            if (bi[w] >= 0 && (piv < 0 || bv[w] > best || (bv[w] == best && bi[w] < piv))) { best = bv[w]; piv = bi[w]; }
-        if (best == 0.0) {
-            if (threadIdx.x == 0) { set_status(status, LAIR_ERR_ZERO_DIAGONAL); bad = 1; }
-            break;
-        }
-        if (piv != k) {
-            for (int c = threadIdx.x; c < n; c += blockDim.x) {
-                double t = D[k * n + c];
-                D[k * n + c] = D[piv * n + c];
-                D[piv * n + c] = t;
+        if (w == 0) {
+            // largest |D[r][k]|, r >= k, ties to the smallest r
+            unsigned long long best = 0;
+            int piv = n;
+            for (int r = k + lane; r < n; r += 32) {
+                const unsigned long long v = (unsigned long long)__double_as_longlong(fabs(D[r * n + k]));
+                if (piv == n || v > best) {
+                    best = v;
+                    piv = r;
+                }
             }
-            if (threadIdx.x == 0) { int t = perm[k]; perm[k] = perm[piv]; perm[piv] = t; }
+            const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
+            const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+            const bool is = piv < n && (unsigned)(best >> 32) == hi && (unsigned)best == lo;
+            piv = (int)__reduce_min_sync(0xffffffffu, is ? (unsigned)piv : 0xffffffffu);
+            if (lane == 0) s_piv = (hi | lo) ? piv : -1;
+            if ((hi | lo) && piv != k) {
+                for (int c = lane; c < n; c += 32) {
+                    const double a = D[k * n + c];
+                    D[k * n + c] = D[piv * n + c];
+                    D[piv * n + c] = a;
+                }
+                if (lane == 0) {
+                    const int a = perm[k];
+                    perm[k] = perm[piv];
+                    perm[piv] = a;
+                }
+            }
         }
         __syncthreads();
+        if (s_piv < 0) {
+            // a singular matrix leaves perm_out at -1, which k_dense_inv_cols reads as "skip"
+            if (t == 0) {
+                set_status(status, LAIR_ERR_ZERO_DIAGONAL);
+                perm_out[0] = -1;
+            }
+            return;
+        }
+        // row r by warp r mod nw; its multiplier by one division for up to 32 of the warp's rows at once
         const double pk = D[k * n + k];
-        for (int r = k + 1 + threadIdx.x; r < n; r += blockDim.x) D[r * n + k] = D[r * n + k] / pk;
-        __syncthreads();
-        const int w = n - k - 1;
-        for (int e = threadIdx.x; e < w * w; e += blockDim.x) {
-            int r = k + 1 + e / w, c = k + 1 + e % w;
-            D[r * n + c] = fma(-D[r * n + k], D[k * n + c], D[r * n + c]);
+        const double *pr = D + k * n;
+        for (int r0 = k + 1 + w; r0 < n; r0 += 32 * nw) {
+            const int rl = r0 + lane * nw;
+            double l = 0.0;
+            if (rl < n) {
+                l = D[rl * n + k];
+                if (l != 0.0) {
+                    l = l / pk;
+                    D[rl * n + k] = l;
+                }
+            }
+            unsigned todo = __ballot_sync(0xffffffffu, l != 0.0);
+            while (todo) {
+                const int b = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const double lr = __shfl_sync(0xffffffffu, l, b);
+                double *row = D + (r0 + b * nw) * n;
+                for (int c = k + 1 + lane; c < n; c += 32) row[c] = fma(-lr, pr[c], row[c]);
+            }
         }
         __syncthreads();
     }
-    __syncthreads();
-    // a singular matrix leaves perm_out at -1, which k_dense_inv_cols reads as "skip"
-    if (threadIdx.x == 0 && bad) perm_out[0] = -1;
-    if (bad) return;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) LU[e] = D[e];
-    for (int i = threadIdx.x; i < n; i += blockDim.x) perm_out[i] = perm[i];
+    for (int e = t; e < n * n; e += T) LU[e] = D[e];
+    for (int i = t; i < n; i += T) perm_out[i] = perm[i];
 }
 
-// columns of the inverse from the factors P A = L U: each warp owns DINV_COLS columns, DINV_ROWS lanes per
-// column take the rows of every substitution step. The device's FP64 pipe serves whole warps, so this keeps
-// the lanes full (a warp per column left most of them idle in the short steps, and a lane per division left 31
-// of 32 idle) and spreads the columns over n / DINV_COLS SMs. Per element the operations and their order are
-// those of the LU solve with e_t as right-hand side: forward x_r -= l_rk x_k, then x_c /= u_cc and
-// x_r -= u_rc x_c for r < c.
-constexpr int DINV_COLS = 4, DINV_ROWS = 32 / DINV_COLS;
+// Columns of the inverse from the factors P A = L U: a CTA of DINV_WARPS warps owns DINV_COLS columns, DINV_COLS lanes
+// next to each other hold one row of them, and the rows of a substitution step are spread over all the warps. Per
+// element the operations and their order are those of the LU solve with e_t as right-hand side: forward
+// x_r -= l_rk x_k, then x_c /= u_cc and x_r -= u_rc x_c for r < c. The steps are a chain of FP64 latencies (65 cycles an
+// fma, several hundred a division) and barriers; the factors are read once per step from shared memory, transposed, so
+// that the rows of a step lie next to each other (they fit up to DENSE_SMEM_N), else from global memory. A step whose
+// x_k is 0 in all columns changes nothing and is passed over (e_t has zeros down to row t of L).
+// Figures: with k_dense_small above.
+constexpr int DINV_COLS = 4, DINV_WARPS = 4, DINV_ROWS = 32 * DINV_WARPS / DINV_COLS;
 
-__global__ void __launch_bounds__(32) k_dense_inv_cols(int n, const double *__restrict__ LU,
-                                                       const int *__restrict__ perm, double *__restrict__ Ainv) {
+template <bool STAGED>
+__global__ void __launch_bounds__(32 * DINV_WARPS) k_dense_inv_cols(int n, const double *__restrict__ LU,
+                                                                    const int *__restrict__ perm,
+                                                                    double *__restrict__ Ainv) {
     extern __shared__ __align__(16) unsigned char smem[];
     double *x = reinterpret_cast<double *>(smem);  // n x DINV_COLS, row-major
+    double *F = x + (size_t)n * DINV_COLS;         // STAGED: F[c][r] = LU[r][c], rows of n + 1 (bank conflicts)
     if (perm[0] < 0) return;
-    const int lane = threadIdx.x, cg = lane / DINV_ROWS, rl = lane % DINV_ROWS;
-    const int t = blockIdx.x * DINV_COLS + cg;
-    for (int r = rl; r < n; r += DINV_ROWS) x[r * DINV_COLS + cg] = perm[r] == t ? 1.0 : 0.0;
-    __syncwarp();
+    const int t = threadIdx.x, cg = t % DINV_COLS, rl = t / DINV_COLS;
+    const int tc = blockIdx.x * DINV_COLS + cg;
+    if (STAGED)
+        for (int e = t; e < n * n; e += blockDim.x) F[(e % n) * (n + 1) + e / n] = LU[e];
+    for (int r = rl; r < n; r += DINV_ROWS) x[r * DINV_COLS + cg] = perm[r] == tc ? 1.0 : 0.0;
+    __syncthreads();
+    auto at = [&](int r, int c) { return STAGED ? F[c * (n + 1) + r] : LU[(size_t)r * n + c]; };
     for (int k = 0; k < n; ++k) {
         const double xk = x[k * DINV_COLS + cg];
-        for (int r = k + 1 + rl; r < n; r += DINV_ROWS)
-            x[r * DINV_COLS + cg] = fma(-LU[(size_t)r * n + k], xk, x[r * DINV_COLS + cg]);
-        __syncwarp();
+        if (__syncthreads_or(xk != 0.0)) {
+            for (int r = k + 1 + rl; r < n; r += DINV_ROWS)
+                x[r * DINV_COLS + cg] = fma(-at(r, k), xk, x[r * DINV_COLS + cg]);
+            __syncthreads();
+        }
     }
     for (int c = n - 1; c >= 0; --c) {
-        const double xc = x[c * DINV_COLS + cg] / LU[(size_t)c * n + c];
-        __syncwarp();
-        if (rl == 0) x[c * DINV_COLS + cg] = xc;
-        for (int r = rl; r < c; r += DINV_ROWS) x[r * DINV_COLS + cg] = fma(-LU[(size_t)r * n + c], xc, x[r * DINV_COLS + cg]);
-        __syncwarp();
+        const double xc = x[c * DINV_COLS + cg] / at(c, c);
+        for (int r = rl; r < c; r += DINV_ROWS) x[r * DINV_COLS + cg] = fma(-at(r, c), xc, x[r * DINV_COLS + cg]);
+        if (rl == 0 && tc < n) Ainv[(size_t)c * n + tc] = xc;
+        __syncthreads();
     }
-    if (t < n)
-        for (int r = rl; r < n; r += DINV_ROWS) Ainv[(size_t)r * n + t] = x[r * DINV_COLS + cg];
 }
 
 bool dense_small(int n) { return n <= DENSE_SMEM_N; }
@@ -1122,12 +1155,10 @@ void launch_dense_setup(const DCsr &A, double *D, int *perm, double *Ainv, int *
     if (n <= DENSE_SMEM_N) {
         size_t bytes = sizeof(double) * (size_t)n * n + sizeof(int) * (size_t)n;
         cudaFuncSetAttribute(k_dense_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        // every column of the elimination costs a few block barriers: fewer warps make them cheaper, and a
-        // coarsest level of a hundred unknowns has little work per column
-        const int tb = n <= 64 ? 128 : 256;
-        k_dense_small<<<1, tb, bytes, s>>>(n, A.rp, A.col, A.val, D, perm, status);
-        k_dense_inv_cols<<<(n + DINV_COLS - 1) / DINV_COLS, 32, sizeof(double) * (size_t)n * DINV_COLS, s>>>(
-            n, D, perm, Ainv);
+        k_dense_small<<<1, 32 * DENSE_WARPS, bytes, s>>>(n, A.rp, A.col, A.val, D, perm, status);
+        const size_t xb = sizeof(double) * ((size_t)n * DINV_COLS + (size_t)n * (n + 1));
+        cudaFuncSetAttribute(k_dense_inv_cols<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xb);
+        k_dense_inv_cols<true><<<(n + DINV_COLS - 1) / DINV_COLS, 32 * DINV_WARPS, xb, s>>>(n, D, perm, Ainv);
         count_launch(2);
         return;
     }
@@ -1138,8 +1169,8 @@ void launch_dense_setup(const DCsr &A, double *D, int *perm, double *Ainv, int *
     // fallback when the four columns' vectors do not fit in shared memory
     const size_t xb = sizeof(double) * (size_t)n * DINV_COLS;
     if (xb <= (size_t)200 * 1024 &&
-        cudaFuncSetAttribute(k_dense_inv_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xb) == cudaSuccess) {
-        k_dense_inv_cols<<<(n + DINV_COLS - 1) / DINV_COLS, 32, xb, s>>>(n, D, perm, Ainv);
+        cudaFuncSetAttribute(k_dense_inv_cols<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xb) == cudaSuccess) {
+        k_dense_inv_cols<false><<<(n + DINV_COLS - 1) / DINV_COLS, 32 * DINV_WARPS, xb, s>>>(n, D, perm, Ainv);
     } else {
         cudaGetLastError();
         k_dense_inverse<<<grid_for(n, 64), 64, 0, s>>>(n, D, perm, Ainv);
