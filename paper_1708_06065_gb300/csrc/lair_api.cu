@@ -2233,6 +2233,7 @@ void lair_free(lair_handle *h) {
     for (auto &p : h->pending) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
     for (auto &p : h->graph_events) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
     for (auto e : h->ev_pool) cudaEventDestroy(e);
+    if (h->col_ev) cudaEventDestroy(h->col_ev);
     if (h->own) cudaStreamDestroy(h->own);
     if (h->h_bat) cudaFreeHost(h->h_bat);
     if (h->h_ring) cudaFreeHost(h->h_ring);

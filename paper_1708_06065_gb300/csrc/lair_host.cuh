@@ -109,6 +109,7 @@ struct lair_handle {
     // outer-iteration work (FP64)
     double *wb = nullptr, *wx = nullptr, *wr = nullptr, *part = nullptr, *dsc = nullptr;
     double *V = nullptr, *Z = nullptr;
+    cudaEvent_t col_ev = nullptr;   // FGMRES: the Hessenberg column has arrived on the host
     int fg_m = 0;
     std::string err;
     long long launches = 0;

@@ -6,21 +6,25 @@
 
 namespace lair {
 
+// one cycle (zero initial guess) of the right-hand side in the finest level's b buffer, result in its x buffer
+static lair_status run_cycle(lair_handle *h, Hier &H) {
+    CU(cudaGraphLaunch(H.graph, h->s));
+    count_launch(H.graph_nodes);
+    h->graph_pending = h->o.timing;
+    return LAIR_OK;
+}
+
 // z = M^{-1} v (one cycle, zero initial guess); v, z: FP64 device vectors of length n0
 lair_status precond(lair_handle *h, Hier &H, const double *v, double *z) {
     Level &L = H.lev[0];
     const int n = L.A.nr;
     if (h->o.precision == LAIR_MIXED) {
         d2f(n, v, L.b32, h->s);
-        CU(cudaGraphLaunch(H.graph, h->s));
-        count_launch(H.graph_nodes);
-        h->graph_pending = h->o.timing;
+        TRY(run_cycle(h, H));
         f2d(n, L.x32[L.xfinal], z, h->s);
     } else {
         CU(cudaMemcpyAsync(L.b64, v, sizeof(double) * n, cudaMemcpyDeviceToDevice, h->s));
-        CU(cudaGraphLaunch(H.graph, h->s));
-        count_launch(H.graph_nodes);
-        h->graph_pending = h->o.timing;
+        TRY(run_cycle(h, H));
         CU(cudaMemcpyAsync(z, L.x64[L.xfinal], sizeof(double) * n, cudaMemcpyDeviceToDevice, h->s));
     }
     return LAIR_OK;
@@ -43,7 +47,7 @@ lair_status ensure_work(lair_handle *h, int n, int m) {
 }
 
 static lair_status norm2_dev(lair_handle *h, int n, const double *v, double *out_dev, double *out_host) {
-    multidot(n, 1, v, n, v, h->part, out_dev, nullptr, h->s);
+    norm2(n, v, h->part, out_dev, h->s);
     if (out_host) {
         CU(cudaMemcpyAsync(h->h_dbl, out_dev, sizeof(double), cudaMemcpyDeviceToHost, h->s));
         CU(cudaStreamSynchronize(h->s));
@@ -80,7 +84,7 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
             int tr = tbegin(h, "outer_residual", (double)A.nnz * 12.0 + (double)n * (4.0 + 16.0 + (mixed ? 4.0 : 8.0)));
             sell_residual(L0.A64, b, x, mixed ? nullptr : L0.b64, mixed ? L0.b32 : nullptr, h->part, h->s);
             tend(h, tr);
-            finish_partials(1, h->part, h->dsc, h->s);
+            finish_residual(h->part, h->dsc, h->s);
             CU(cudaMemcpyAsync(h->h_dbl, h->dsc, sizeof(double), cudaMemcpyDeviceToHost, h->s));
             CU(cudaStreamSynchronize(h->s));
 
@@ -100,10 +104,16 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
     } else {
         double *V = h->V, *Z = h->Z;
         std::vector<double> Hm((size_t)(m + 1) * m, 0.0), cs(m), sn(m), g(m + 1), hc(m + 2), y(m + 1);
-        // device scalars: |r|^2 at 1, Hessenberg column at 8 (32), the two CGS2 projections at 48 (64), y at 112 (32)
-        double *hsum = h->dsc + 8, *hbuf = h->dsc + 48, *nrm = h->dsc + 1, *ydev = h->dsc + 112;
+        // device scalars: |r|^2 or |w|^2 at 7, Hessenberg column behind it (32), the two CGS2 projections at 48 (64), y
+        // at 112 (32)
+        double *nrm = h->dsc + 7, *hsum = nrm + 1, *hbuf = h->dsc + 48, *ydev = h->dsc + 112;
+        auto scale = [&](double *v) {   // v <- v / |v|, also into the cycle's right-hand side
+            if (mixed) scale_by_norm<float>(n, v, nrm, L0.b32, h->s);
+            else scale_by_norm<double>(n, v, nrm, L0.b64, h->s);
+        };
+        if (!h->col_ev) CU(cudaEventCreateWithFlags(&h->col_ev, cudaEventDisableTiming));
         sell_residual(L0.A64, b, x, V, nullptr, h->part, h->s);
-        finish_partials(1, h->part, nrm, h->s);
+        finish_residual(h->part, nrm, h->s);
         CU(cudaMemcpyAsync(h->h_dbl, nrm, sizeof(double), cudaMemcpyDeviceToHost, h->s));
         CU(cudaStreamSynchronize(h->s));
 
@@ -112,34 +122,33 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
         rel = beta / bn;
         hist(rel);
         while (std::isfinite(rel) && rel > tol && it < max_iter) {
-            scale_by_norm(n, V, nrm, V, h->s);
+            scale(V);
             std::fill(g.begin(), g.end(), 0.0);
             g[0] = beta;
             int jdone = 0;
             for (int j = 0; j < m && it < max_iter; ++j) {
-                double *vj = V + (size_t)j * n, *zj = Z + (size_t)j * n, *w = V + (size_t)(j + 1) * n;
-                TRY(precond(h, H, vj, zj));
+                double *zj = Z + (size_t)j * n, *w = V + (size_t)(j + 1) * n;
+                TRY(run_cycle(h, H));   // of v_j
                 ++it;
                 int ts = tbegin(h, "outer_spmv", bytes_spmv(A, 8.0));
-                sell_spmv<double>(L0.A64, zj, w, h->s);
+                if (mixed) sell_spmv_keep<float>(L0.A64, L0.x32[L0.xfinal], zj, w, h->s);
+                else sell_spmv_keep<double>(L0.A64, L0.x64[L0.xfinal], zj, w, h->s);
                 tend(h, ts);
-                CU(cudaMemsetAsync(hsum, 0, sizeof(double) * (j + 1), h->s));
                 int to = tbegin(h, "outer_cgs2", 8.0 * n * (3.0 * (j + 2) + 4.0));
-                cgs_pass(1, n, j + 1, V, n, nullptr, w, h->part, h->s);
-                finish_partials_acc(j + 1, h->part, hbuf, hsum, h->s);
-                cgs_pass(2, n, j + 1, V, n, hbuf, w, h->part, h->s);
-                finish_partials_acc(j + 1, h->part, hbuf + 32, hsum, h->s);
-                cgs_pass(3, n, j + 1, V, n, hbuf + 32, w, h->part, h->s);
-                finish_partials(1, h->part, nrm, h->s);
-                scale_by_norm(n, w, nrm, w, h->s);
+                cgs2(n, j + 1, V, n, w, h->part, hbuf, hbuf + 32, hsum, nrm, h->s);
+                // the host reads the column and goes on while w is being scaled
+                CU(cudaMemcpyAsync(h->h_dbl, nrm, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, h->s));
+                CU(cudaEventRecord(h->col_ev, h->s));
+                scale(w);
                 tend(h, to);
-                CU(cudaMemcpyAsync(h->h_dbl, hsum, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, h->s));
-                CU(cudaMemcpyAsync(h->h_dbl + 40, nrm, sizeof(double), cudaMemcpyDeviceToHost, h->s));
-                CU(cudaStreamSynchronize(h->s));
-
-                flush_timers(h);
-                for (int k = 0; k <= j; ++k) hc[k] = h->h_dbl[k];
-                double hn = std::sqrt(h->h_dbl[40]);
+                if (h->o.timing) {
+                    CU(cudaStreamSynchronize(h->s));
+                    flush_timers(h);
+                } else {
+                    CU(cudaEventSynchronize(h->col_ev));
+                }
+                for (int k = 0; k <= j; ++k) hc[k] = h->h_dbl[k + 1];
+                double hn = std::sqrt(h->h_dbl[0]);
                 hc[j + 1] = hn;
                 for (int k = 0; k < j; ++k) {
                     double t = cs[k] * hc[k] + sn[k] * hc[k + 1];
@@ -166,7 +175,7 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
             CU(cudaMemcpyAsync(ydev, y.data(), sizeof(double) * jdone, cudaMemcpyHostToDevice, h->s));
             add_combo(n, jdone, Z, n, ydev, x, h->s);
             sell_residual(L0.A64, b, x, V, nullptr, h->part, h->s);
-            finish_partials(1, h->part, nrm, h->s);
+            finish_residual(h->part, nrm, h->s);
             CU(cudaMemcpyAsync(h->h_dbl, nrm, sizeof(double), cudaMemcpyDeviceToHost, h->s));
             CU(cudaStreamSynchronize(h->s));
 
@@ -382,6 +391,11 @@ lair_status solve_batched_fgmres(lair_handle *h, Hier &H, const double *b, doubl
     c.max_iter = max_iter;
     SegTiles sta = h->segt;   // the Arnoldi kernels skip the tiles of systems that are not running
     sta.active = c.run;
+    const bool mixed = h->o.precision == LAIR_MIXED;
+    auto scale = [&](double *v) {   // v_q <- v_q / |v_q| of the running systems, also into the cycle's right-hand side
+        if (mixed) seg_scale<float>(sta, v, nrm, L0.b32, h->s);
+        else seg_scale<double>(sta, v, nrm, L0.b64, h->s);
+    };
     seg_norm2(h->segt, b, nrm, h->s);
     bat_bnorm(nseg, nrm, const_cast<double *>(c.bn), h->s);
     CU(cudaMemsetAsync(c.its, 0, sizeof(int) * nseg, h->s));
@@ -398,24 +412,24 @@ lair_status solve_batched_fgmres(lair_handle *h, Hier &H, const double *b, doubl
         ++step;
         flush_timers(h);
         if (running == 0) break;
-        seg_scale(sta, V, nrm, V, h->s);
+        scale(V);
         const long long first = step;
         for (int j = 0; j < m; ++j) {
             if (step - first >= lair_handle::LAG) {
                 TRY(ring_read(h, step - lair_handle::LAG, &running));
                 if (running == 0) break;
             }
-            double *vj = V + (size_t)j * n, *zj = Z + (size_t)j * n, *w = V + (size_t)(j + 1) * n;
-            TRY(precond(h, H, vj, zj));
+            double *zj = Z + (size_t)j * n, *w = V + (size_t)(j + 1) * n;
+            TRY(run_cycle(h, H));   // of v_j
             int ts = tbegin(h, "outer_spmv", bytes_spmv(A, 8.0));
-            sell_spmv<double>(L0.A64, zj, w, h->s);
+            if (mixed) sell_spmv_keep<float>(L0.A64, L0.x32[L0.xfinal], zj, w, h->s);
+            else sell_spmv_keep<double>(L0.A64, L0.x64[L0.xfinal], zj, w, h->s);
             tend(h, ts);
-            CU(cudaMemsetAsync(hsum, 0, sizeof(double) * (size_t)nseg * HS, h->s));
             // CGS2 in three streaming passes over V: dots; update and dots; update and norm
             seg_cgs_pass(sta, 1, j + 1, V, n, HS, nullptr, w, hbuf, hsum, h->s);
             seg_cgs_pass(sta, 2, j + 1, V, n, HS, hbuf, w, hbuf, hsum, h->s);
             seg_cgs_pass(sta, 3, j + 1, V, n, HS, hbuf, w, nrm, nullptr, h->s);
-            seg_scale(sta, w, nrm, w, h->s);
+            scale(w);
             CU(cudaMemsetAsync(ring_slot(h, step), 0, sizeof(int), h->s));
             bat_fg_givens(c, j, hsum, nrm, ring_slot(h, step), h->s);
             TRY(ring_post(h, step));

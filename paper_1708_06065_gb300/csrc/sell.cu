@@ -384,15 +384,17 @@ struct RowHead {
             w[k] = k < len ? __ldg(val + base + 32 * k) : T(0);
         }
     }
-    __device__ __forceinline__ T sum(const SellView &v, const T *x) const {
+    // (x in X: T, or FP32 widened to T)
+    template <class X>
+    __device__ __forceinline__ T sum(const SellView &v, const X *x) const {
         T acc = T(0);
         {
-            T xv[NB];
+            X xv[NB];
 #pragma unroll
-            for (int k = 0; k < NB; ++k) xv[k] = k < len ? x[c[k]] : T(0);
+            for (int k = 0; k < NB; ++k) xv[k] = k < len ? x[c[k]] : X(0);
 #pragma unroll
             for (int k = 0; k < NB; ++k)
-                if (k < len) acc = fma(w[k], xv[k], acc);
+                if (k < len) acc = fma(w[k], (T)xv[k], acc);
         }
         const T *val = static_cast<const T *>(v.val);
         for (int j = NB; j < len; j += NB) {
@@ -405,7 +407,7 @@ struct RowHead {
             }
 #pragma unroll
             for (int k = 0; k < NB; ++k)
-                if (j + k < len) acc = fma(ww[k], x[cc[k]], acc);
+                if (j + k < len) acc = fma(ww[k], (T)x[cc[k]], acc);
         }
         return acc;
     }
@@ -829,8 +831,64 @@ void launch_p1_cols(int n, const int *rp, const int *col, int *p1col, cudaStream
     count_launch();
 }
 
+// The outer iteration's product y = A z with z = the cycle's result x (FP32, widened exactly, or FP64), which the
+// kernel also writes out: one launch instead of a conversion and a product, and in mixed precision the gathers read
+// half the bytes. The arithmetic of k_sell_spmv<double>.
+template <class T>
+__global__ void __launch_bounds__(256) k_sell_spmv_keep(SellView v, const T *x, double *z, double *y) {
+    pdl_enter();
+    const int *__restrict__ sptr = v.slice_ptr;
+    const int *__restrict__ scol = v.col;
+    const double *__restrict__ sval = static_cast<const double *>(v.val);
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < v.nrows; q += gridDim.x * blockDim.x) {
+        const int sl = q >> 5;
+        bool on = true;
+        if (v.run) {
+            const int sy = v.slice_sys[sl];
+            on = sy < 0 || v.run[sy];
+        }
+        const int a = __ldg(sptr + sl), base = a + (q & 31);
+        const int len = on ? (__ldg(sptr + sl + 1) - a) >> 5 : 0;   // a stopped system: y = 0
+        const int i = __ldg(v.row + q);
+        double acc = 0.0;
+#pragma unroll 4
+        for (int j = 0; j < len; ++j) acc = fma(__ldcs(sval + base + 32 * j), (double)x[__ldcs(scol + base + 32 * j)], acc);
+        y[i] = acc;
+        z[i] = (double)x[i];
+    }
+}
+
+template <class T, int NB>
+__global__ void __launch_bounds__(WAVE_THREADS) k_sell_spmv_keep_wave(SellView v, const T *x, double *z, double *y) {
+    pdl_launch_next();
+    const int u = blockIdx.x * WAVE_THREADS + threadIdx.x;
+    RowHead<double, NB> h;
+    if (u < ((v.nrows + 31) & ~31)) h.load(v, u, v.nrows);
+    pdl_wait_previous();
+    const double acc = h.sum(v, x);
+    if (h.i >= 0) {
+        y[h.i] = acc;
+        z[h.i] = (double)x[h.i];
+    }
+}
+
+template <class T>
+void sell_spmv_keep(const SellView &v, const T *x, double *z, double *y, cudaStream_t s) {
+    if (v.nrows <= 0) return;
+    if (v.nrows <= one_wave_rows<double>()) {
+        const int grid = (v.nrows + WAVE_THREADS - 1) / WAVE_THREADS;
+        if (v.long_rows) launch_pdl(k_sell_spmv_keep_wave<T, 16>, grid, WAVE_THREADS, 0, s, v, x, z, y);
+        else launch_pdl(k_sell_spmv_keep_wave<T, 8>, grid, WAVE_THREADS, 0, s, v, x, z, y);
+    } else {
+        launch_pdl(k_sell_spmv_keep<T>, grid_for(v.nrows, 256, device_sms() * 16), 256, 0, s, v, x, z, y);
+    }
+    count_launch();
+}
+template void sell_spmv_keep<float>(const SellView &, const float *, double *, double *, cudaStream_t);
+template void sell_spmv_keep<double>(const SellView &, const double *, double *, double *, cudaStream_t);
+
 // r = b - A x over all rows of an FP64 view of A (r and its FP32 copy each optional), and the block partial
-// of |r|^2 in part[blockIdx.x] (gridDim.x = RED_PARTS blocks, summed by finish_partials)
+// of |r|^2 in part[blockIdx.x] (gridDim.x = RED_PARTS blocks, summed by finish_residual)
 constexpr int RES_THREADS = 512;
 
 __global__ void __launch_bounds__(RES_THREADS) k_sell_residual(SellView v, const double *__restrict__ b,

@@ -186,25 +186,20 @@ void launch_to_f32(long long n, const double *a, float *b, cudaStream_t s);
 void launch_dense_setup(const DCsr &A, double *D, int *perm, double *Ainv, int *status, cudaStream_t s);
 
 // ---- solve_kernels.cu -----------------------------------------------------------------
-template <class T> void spmv(const DCsr &A, const T *x, T *y, cudaStream_t s);
-template <class T>
-void sweep(const DCsr &A, const int8_t *cf, int target, const T *dinv, const T *b, const T *x, T *xo, cudaStream_t s);
 template <class T> void dense_apply(int n, const double *Ainv, const T *b, T *y, cudaStream_t s);
 constexpr int RED_PARTS = 152 * 4;
-void residual(const DCsr &A, const double *b, const double *x, double *r, float *r32, double *part, cudaStream_t s);
-// the same over an FP64 sliced-ELL view of all rows (RED_PARTS block partials)
+// r = b - A x over an FP64 sliced-ELL view of all rows (r and its FP32 copy optional); |r|^2 as RED_PARTS block partials
 void sell_residual(const SellView &v, const double *b, const double *x, double *r, float *r32, double *part,
                    cudaStream_t s);
-void multidot(int n, int m, const double *X, long long ldx, const double *y, double *part, double *out, double *acc,
-              cudaStream_t s);
-void finish_partials(int m, const double *part, double *out, cudaStream_t s);
-void finish_partials_acc(int m, const double *part, double *out, double *acc, cudaStream_t s);
-// one pass (1, 2 or 3) of CGS2 of w against the m <= 32 columns of X; block partials in part
-void cgs_pass(int pass, int n, int m, const double *X, long long ldx, const double *h, double *w, double *part,
-              cudaStream_t s);
-void sub_combo(int n, int m, const double *X, long long ldx, const double *h, double *w, cudaStream_t s);
+void finish_residual(const double *part, double *out, cudaStream_t s);   // the sum of sell_residual's partials
+void norm2(int n, const double *v, double *part, double *out, cudaStream_t s);
+// CGS2 of w against the m <= 32 columns of X: the sums of both projections to hsum, the new |w|^2 to nrm; part, h1 and
+// h2 (32 each): scratch
+void cgs2(int n, int m, const double *X, long long ldx, double *w, double *part, double *h1, double *h2, double *hsum,
+          double *nrm, cudaStream_t s);
 void add_combo(int n, int m, const double *Z, long long ldz, const double *y, double *x, cudaStream_t s);
-void scale_by_norm(int n, const double *v, const double *nrm2, double *out, cudaStream_t s);
+// v <- v / sqrt(*nrm2), and c = the same in T
+template <class T> void scale_by_norm(int n, double *v, const double *nrm2, T *c, cudaStream_t s);
 void d2f(int n, const double *a, float *b, cudaStream_t s);
 void f2d(int n, const float *a, double *b, cudaStream_t s);
 void axpy_f(int n, const float *e, double *x, cudaStream_t s);
@@ -234,6 +229,8 @@ void launch_sell_fill_multi(const SellDesc *d, int p0, int p1, int lin_beg, int 
 // the largest view that the one-wave kernels take
 template <class T> long long one_wave_rows() { return (long long)device_sms() * (WAVE_BYTES_PER_SM / (int)sizeof(T)); }
 template <class T> void sell_spmv(const SellView &v, const T *x, T *y, cudaStream_t s);
+// y = A x for an FP64 view of all rows of A and an x in T, and z = x in FP64
+template <class T> void sell_spmv_keep(const SellView &v, const T *x, double *z, double *y, cudaStream_t s);
 template <class T>
 void sell_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const T *x, T *xo, cudaStream_t s);
 // x = P x_c for a P with at most one entry per row, every entry 1 (one-point interpolation), from its dense
@@ -306,13 +303,13 @@ void seg_norm2(const SegTiles &st, const double *v, double *norm2, cudaStream_t 
 template <class T>
 void seg_axpy(const SegTiles &st, const uint8_t *active, const T *e, double *x, cudaStream_t s);
 // one pass of the batched CGS2 step (see k_tile_cgs) over the m <= 31 columns of X, then the per-system sums:
-// passes 1 and 2 write the m dots of every running system to out[q * hs + k] and add them to acc[q * hs + k],
+// passes 1 and 2 write the m dots of every running system to out[q * hs + k] and set / add to acc[q * hs + k],
 // pass 3 writes the squared norm of the new w to out[q]
 void seg_cgs_pass(const SegTiles &st, int pass, int m, const double *X, long long ldx, int hs, const double *h, double *w,
                   double *out, double *acc, cudaStream_t s);
 void seg_add_combo(const SegTiles &st, const int *cnt, const double *Z, long long ldz, int hs, const double *y, double *x,
                    cudaStream_t s);
-void seg_scale(const SegTiles &st, const double *v, const double *nrm2, double *out, cudaStream_t s);
+template <class T> void seg_scale(const SegTiles &st, double *v, const double *nrm2, T *c, cudaStream_t s);
 void gather_int(int m, const int *idx, const int *src, int *out, cudaStream_t s);
 // device-side state of the batched outer loops (one entry per system; see solve_kernels.cu)
 constexpr int BATCH_HS = 32;      // Hessenberg column stride: restart lengths up to 31

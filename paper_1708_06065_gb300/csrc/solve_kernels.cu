@@ -2,122 +2,9 @@
 // x = P x_c, Jacobi F/C sweeps x_i <- x_i + d_i (b_i - A_i x) (Eq. (2.4)), the dense
 // coarsest solve, and the FP64 outer-iteration kernels (residual, norms, block dots
 // for classical Gram-Schmidt, updates).
-//
-// Sparse rows are processed by groups of G consecutive lanes (G = 1, 2, 4, 8, 16 or
-// 32, picked from the average row length); group lanes stride over the row so that
-// consecutive lanes load consecutive column indices and values, and the partial sums
-// are combined by xor-shuffles inside the group. All of these kernels are bound by
-// HBM bandwidth on the large levels.
 #include "setup_kernels.cuh"
 
 namespace lair {
-
-template <int G, class T>
-__device__ __forceinline__ T group_sum(T v) {
-#pragma unroll
-    for (int o = G / 2; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// y = A x  (also R b and P x_c)
-template <int G, class T>
-__global__ void __launch_bounds__(256) k_spmv(int nr, const int *__restrict__ rp, const int *__restrict__ col,
-                                             const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y) {
-    const int gl = threadIdx.x & (G - 1);
-    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    const long long lane = threadIdx.x & 31;
-    for (long long base = tid; base - lane < (long long)nr * G; base += stride) {  // warp-uniform trip count
-        int i = (int)(base / G);
-        T acc = T(0);
-        if (i < nr) {
-            int b = __ldg(rp + i), e = __ldg(rp + i + 1);
-            for (int k = b + gl; k < e; k += G) acc = fma(__ldg(val + k), __ldg(x + __ldg(col + k)), acc);
-        }
-        acc = group_sum<G>(acc);
-        if (i < nr && gl == 0) y[i] = acc;
-    }
-}
-
-// one Jacobi sweep over the points with cf == target; all other points are copied
-template <int G, class T>
-__global__ void __launch_bounds__(256) k_sweep(int nr, const int *__restrict__ rp, const int *__restrict__ col,
-                                              const T *__restrict__ val, const int8_t *__restrict__ cf, int target,
-                                              const T *__restrict__ dinv, const T *__restrict__ b,
-                                              const T *__restrict__ x, T *__restrict__ xo) {
-    const int gl = threadIdx.x & (G - 1);
-    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    const long long lane = threadIdx.x & 31;
-    for (long long base = tid; base - lane < (long long)nr * G; base += stride) {  // warp-uniform trip count
-        int i = (int)(base / G);
-        bool act = i < nr && cf[i] == target;
-        T acc = T(0);
-        if (act) {
-            int bb = __ldg(rp + i), e = __ldg(rp + i + 1);
-            for (int k = bb + gl; k < e; k += G) acc = fma(__ldg(val + k), __ldg(x + __ldg(col + k)), acc);
-        }
-        acc = group_sum<G>(acc);
-        if (i < nr && gl == 0) xo[i] = act ? fma(dinv[i], b[i] - acc, x[i]) : x[i];
-    }
-}
-
-template <class T>
-static int pick_group(const DCsr &A) {
-    double avg = A.nr > 0 ? (double)A.nnz / A.nr : 1.0;
-    if (avg <= 1.5) return 1;
-    if (avg <= 3.0) return 2;
-    if (avg <= 10.0) return 4;
-    if (avg <= 24.0) return 8;
-    if (avg <= 48.0) return 16;
-    return 32;
-}
-
-template <class T>
-static const T *vals_of(const DCsr &A);
-template <> const double *vals_of<double>(const DCsr &A) { return A.val; }
-template <> const float *vals_of<float>(const DCsr &A) { return A.val32; }
-
-template <class T>
-void spmv(const DCsr &A, const T *x, T *y, cudaStream_t s) {
-    if (A.nr == 0) return;
-    int G = pick_group<T>(A);
-    int grid = grid_for((long long)A.nr * G, 256, device_sms() * 16);
-    const T *v = vals_of<T>(A);
-    switch (G) {
-        case 1: k_spmv<1, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, x, y); break;
-        case 2: k_spmv<2, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, x, y); break;
-        case 4: k_spmv<4, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, x, y); break;
-        case 8: k_spmv<8, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, x, y); break;
-        case 16: k_spmv<16, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, x, y); break;
-        default: k_spmv<32, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, x, y); break;
-    }
-    count_launch();
-}
-
-template <class T>
-void sweep(const DCsr &A, const int8_t *cf, int target, const T *dinv, const T *b, const T *x, T *xo, cudaStream_t s) {
-    if (A.nr == 0) return;
-    int G = pick_group<T>(A);
-    int grid = grid_for((long long)A.nr * G, 256, device_sms() * 16);
-    const T *v = vals_of<T>(A);
-    switch (G) {
-        case 1: k_sweep<1, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, cf, target, dinv, b, x, xo); break;
-        case 2: k_sweep<2, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, cf, target, dinv, b, x, xo); break;
-        case 4: k_sweep<4, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, cf, target, dinv, b, x, xo); break;
-        case 8: k_sweep<8, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, cf, target, dinv, b, x, xo); break;
-        case 16: k_sweep<16, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, cf, target, dinv, b, x, xo); break;
-        default: k_sweep<32, T><<<grid, 256, 0, s>>>(A.nr, A.rp, A.col, v, cf, target, dinv, b, x, xo); break;
-    }
-    count_launch();
-}
-
-template void spmv<double>(const DCsr &, const double *, double *, cudaStream_t);
-template void spmv<float>(const DCsr &, const float *, float *, cudaStream_t);
-template void sweep<double>(const DCsr &, const int8_t *, int, const double *, const double *, const double *, double *,
-                            cudaStream_t);
-template void sweep<float>(const DCsr &, const int8_t *, int, const float *, const float *, const float *, float *,
-                           cudaStream_t);
 
 // coarsest level: y = Ainv b (dense, FP64), with the input/output in T
 template <class T>
@@ -145,140 +32,110 @@ template void dense_apply<float>(int, const double *, const float *, float *, cu
 // ---------------------------------------------------------------------------------------
 // FP64 outer iteration
 // ---------------------------------------------------------------------------------------
-constexpr int RED_BLOCKS = 152 * 4;
 constexpr int RED_THREADS = 256;
 
-// r = b - A x (FP64, one thread per row... group of G lanes), optional float copy, block partials of |r|^2
-template <int G>
-__global__ void __launch_bounds__(RED_THREADS) k_residual(int nr, const int *__restrict__ rp, const int *__restrict__ col,
-                                                          const double *__restrict__ val, const double *__restrict__ b,
-                                                          const double *__restrict__ x, double *__restrict__ r,
-                                                          float *__restrict__ r32, double *__restrict__ part) {
-    __shared__ double red[RED_THREADS / 32];
-    const int gl = threadIdx.x & (G - 1);
-    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    double ss = 0.0;
-    const long long lane = threadIdx.x & 31;
-    for (long long base = tid; base - lane < (long long)nr * G; base += stride) {  // warp-uniform trip count
-        int i = (int)(base / G);
-        double acc = 0.0;
-        if (i < nr)
-            for (int k = __ldg(rp + i) + gl; k < __ldg(rp + i + 1); k += G) acc = fma(__ldg(val + k), __ldg(x + __ldg(col + k)), acc);
-        acc = group_sum<G>(acc);
-        if (i < nr && gl == 0) {
-            double ri = b[i] - acc;
-            r[i] = ri;
-            if (r32) r32[i] = (float)ri;
-            ss = fma(ri, ri, ss);
-        }
-    }
-    ss = warp_sum(ss);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) t += red[w];
-        part[blockIdx.x] = t;
-    }
-}
+// ---------------------------------------------------------------------------------------
+// Reductions of the outer iteration. A warp FP64 instruction occupies an SM for 19 cycles whatever its lanes hold, so
+// what a reduction costs is its number of such instructions, not its bytes: five butterfly additions per value and
+// warp, over many warps with one or two elements a thread, took several times the products themselves. So the kernels
+// run few blocks with many elements per thread (red_blocks), and a warp reduces eight values together: each half,
+// quarter and eighth of the warp goes on with its own values, nine additions for eight values instead of forty.
+// Block partials go to part[k * RED_PARTS + block]; k_finish sums them in a fixed order.
+// ---------------------------------------------------------------------------------------
 
-void residual(const DCsr &A, const double *b, const double *x, double *r, float *r32, double *part, cudaStream_t s) {
-    int G = pick_group<double>(A);
-    switch (G) {
-        case 1: k_residual<1><<<RED_BLOCKS, RED_THREADS, 0, s>>>(A.nr, A.rp, A.col, A.val, b, x, r, r32, part); break;
-        case 2: k_residual<2><<<RED_BLOCKS, RED_THREADS, 0, s>>>(A.nr, A.rp, A.col, A.val, b, x, r, r32, part); break;
-        case 4: k_residual<4><<<RED_BLOCKS, RED_THREADS, 0, s>>>(A.nr, A.rp, A.col, A.val, b, x, r, r32, part); break;
-        case 8: k_residual<8><<<RED_BLOCKS, RED_THREADS, 0, s>>>(A.nr, A.rp, A.col, A.val, b, x, r, r32, part); break;
-        case 16: k_residual<16><<<RED_BLOCKS, RED_THREADS, 0, s>>>(A.nr, A.rp, A.col, A.val, b, x, r, r32, part); break;
-        default: k_residual<32><<<RED_BLOCKS, RED_THREADS, 0, s>>>(A.nr, A.rp, A.col, A.val, b, x, r, r32, part); break;
-    }
-    count_launch();
+// the warp's sums of v[0..8); value k is complete in the four lanes whose bits 4, 3 and 2 are bits 2, 1 and 0 of k
+__device__ __forceinline__ double warp_sum8(const double (&v)[8]) {
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, q = lane & 8, e = lane & 4;
+    double a[4], c[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = (h ? v[k + 4] : v[k]) + __shfl_xor_sync(0xffffffffu, h ? v[k] : v[k + 4], 16);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) c[k] = (q ? a[k + 2] : a[k]) + __shfl_xor_sync(0xffffffffu, q ? a[k] : a[k + 2], 8);
+    double r = (e ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, e ? c[0] : c[1], 4);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    return r + __shfl_xor_sync(0xffffffffu, r, 1);
 }
+__device__ __forceinline__ int warp_sum8_index() { return (threadIdx.x >> 2) & 7; }
 
-// block partials of sum_i x_i y_i for vectors x_k (stride ldx) against y, MD vectors per launch:
-// part[k * RED_BLOCKS + block] for k = k0 .. k0 + m - 1
-constexpr int MD = 8;
-__global__ void __launch_bounds__(RED_THREADS) k_multidot(int n, int k0, int m, const double *__restrict__ X, long long ldx,
-                                                          const double *__restrict__ y, double *__restrict__ part) {
-    __shared__ double red[RED_THREADS / 32][MD];
-    double acc[MD];
+// part[k * RED_PARTS + blockIdx.x] = the block's sum of v[k], k < m <= MM
+template <int MM>
+__device__ __forceinline__ void block_partials(const double (&v)[MM], int m, double *part) {
+    static_assert(MM % 8 == 0, "values in groups of eight");
+    __shared__ double red[RED_THREADS / 32][MM];
 #pragma unroll
-    for (int k = 0; k < MD; ++k) acc[k] = 0.0;
-    const double *Xk = X + (long long)k0 * ldx;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        double yi = y[i];
+    for (int g = 0; g < MM; g += 8)
+        if (g < m) {
+            double w[8];
 #pragma unroll
-        for (int k = 0; k < MD; ++k)
-            if (k < m) acc[k] = fma(Xk[k * ldx + i], yi, acc[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < MD; ++k) {
-        if (k < m) {
-            double v = warp_sum(acc[k]);
-            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
+            for (int k = 0; k < 8; ++k) w[k] = v[g + k];
+            const double r = warp_sum8(w);
+            if ((threadIdx.x & 3) == 0) red[threadIdx.x >> 5][g + warp_sum8_index()] = r;
         }
-    }
     __syncthreads();
-    if (threadIdx.x < m) {
+    if ((int)threadIdx.x < m) {
         double t = 0.0;
         for (int w = 0; w < RED_THREADS / 32; ++w) t += red[w][threadIdx.x];
-        part[(k0 + threadIdx.x) * RED_BLOCKS + blockIdx.x] = t;
+        part[threadIdx.x * RED_PARTS + blockIdx.x] = t;
     }
 }
 
-// out[k] = sum of the RED_BLOCKS partials of vector k (fixed order); if acc != NULL, acc[k] += out[k]
-__global__ void k_finish(int m, const double *__restrict__ part, double *__restrict__ out, double *__restrict__ acc) {
-    int k = blockIdx.x;
+// blocks of a reduction over n elements: two or more elements per thread, at most two blocks per SM
+static int red_blocks(int n) {
+    const int want = (n + RED_THREADS * 2 - 1) / (RED_THREADS * 2), most = 2 * device_sms();
+    const int g = want < most ? (want > 0 ? want : 1) : most;
+    return g < RED_PARTS ? g : RED_PARTS;
+}
+
+// out[k] = sum of the nb partials of vector k (fixed order); acc (if any): acc[k] = out[k] when first, else += out[k]
+__global__ void __launch_bounds__(128) k_finish(int m, int nb, const double *part, double *out, double *acc, int first) {
+    pdl_enter();
+    const int k = blockIdx.x;
     if (k >= m) return;
-    __shared__ double red[32];
+    __shared__ double red[4];
     double t = 0.0;
-    for (int b = threadIdx.x; b < RED_BLOCKS; b += blockDim.x) t += part[k * RED_BLOCKS + b];
+    for (int b = threadIdx.x; b < nb; b += 128) t += part[k * RED_PARTS + b];
     t = warp_sum(t);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double u = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) u += red[w];
+        const double u = ((red[0] + red[1]) + red[2]) + red[3];
         out[k] = u;
-        if (acc) acc[k] += u;
+        if (acc) acc[k] = first ? u : acc[k] + u;
     }
 }
 
-void multidot(int n, int m, const double *X, long long ldx, const double *y, double *part, double *out, double *acc,
-              cudaStream_t s) {
-    for (int k0 = 0; k0 < m; k0 += MD) {
-        int mm = m - k0 < MD ? m - k0 : MD;
-        k_multidot<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, k0, mm, X, ldx, y, part);
-        count_launch();
+static void finish(int m, int nb, const double *part, double *out, double *acc, int first, cudaStream_t s) {
+    launch_pdl(k_finish, m, 128, 0, s, m, nb, part, out, acc, first);
+    count_launch();
+}
+
+void finish_residual(const double *part, double *out, cudaStream_t s) {
+    finish(1, RED_PARTS, part, out, nullptr, 1, s);
+}
+
+// |v|^2 as block partials
+__global__ void __launch_bounds__(RED_THREADS) k_norm2(int n, const double *v, double *part) {
+    pdl_enter();
+    double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (; i + 3 * stride < n; i += 4 * stride) {
+        double x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = v[i + k * stride];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[0] = fma(x[k], x[k], acc[0]);
     }
-    k_finish<<<m, 256, 0, s>>>(m, part, out, acc);
-    count_launch();
+    for (; i < n; i += stride) acc[0] = fma(v[i], v[i], acc[0]);
+    block_partials<8>(acc, 1, part);
 }
 
-void finish_partials(int m, const double *part, double *out, cudaStream_t s) {
-    k_finish<<<m, 256, 0, s>>>(m, part, out, nullptr);
+void norm2(int n, const double *v, double *part, double *out, cudaStream_t s) {
+    const int nb = red_blocks(n);
+    launch_pdl(k_norm2, nb, RED_THREADS, 0, s, n, v, part);
     count_launch();
-}
-
-void finish_partials_acc(int m, const double *part, double *out, double *acc, cudaStream_t s) {
-    k_finish<<<m, 256, 0, s>>>(m, part, out, acc);
-    count_launch();
-}
-
-// w -= sum_k h_k X_k (h on the device)
-__global__ void k_sub_combo(int n, int m, const double *__restrict__ X, long long ldx, const double *__restrict__ h,
-                            double *__restrict__ w) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        double v = w[i];
-        for (int k = 0; k < m; ++k) v = fma(-h[k], X[k * ldx + i], v);
-        w[i] = v;
-    }
-}
-
-void sub_combo(int n, int m, const double *X, long long ldx, const double *h, double *w, cudaStream_t s) {
-    k_sub_combo<<<grid_for(n, 256, device_sms() * 8), 256, 0, s>>>(n, m, X, ldx, h, w);
-    count_launch();
+    finish(1, nb, part, out, nullptr, 1, s);
 }
 
 // x += sum_k y_k Z_k (y on the device)
@@ -303,36 +160,23 @@ void add_combo(int n, int m, const double *Z, long long ldz, const double *y, do
 //   pass 2: w <- w - sum_k h1_k X_k, then part_k = X_k . w (the new w)
 //   pass 3: w <- w - sum_k h2_k X_k, then part_0 = w . w
 // Each thread loads X_k[i] once per pass and keeps it in registers for both of its uses.
-// The w update accumulates fma(-h_k, X_k[i], .) in ascending k.
+// The w update accumulates fma(-h_k, X_k[i], .) in ascending k. Bound by the FP64 units (4 m n fma a step).
 // ---------------------------------------------------------------------------------------
-template <int MM>
-__device__ __forceinline__ void block_partials(const double (&acc)[MM], int m, double *part) {
-    __shared__ double red[RED_THREADS / 32][MM];
-#pragma unroll
-    for (int k = 0; k < MM; ++k)
-        if (k < m) {
-            const double v = warp_sum(acc[k]);
-            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
-        }
-    __syncthreads();
-    if ((int)threadIdx.x < m) {
-        double t = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) t += red[w][threadIdx.x];
-        part[threadIdx.x * RED_BLOCKS + blockIdx.x] = t;
-    }
-}
-
 template <int MM, int PASS>
-__global__ void __launch_bounds__(RED_THREADS, MM <= 8 ? RED_BLOCKS / 152 : 1) k_cgs_pass(int n, int m, const double *__restrict__ X, long long ldx,
-                                                          const double *__restrict__ h, double *__restrict__ w,
-                                                          double *__restrict__ part) {
-    double acc[MM];
-    double hk[MM];
+__global__ void __launch_bounds__(RED_THREADS, MM <= 16 ? 2 : 1) k_cgs_pass(int n, int m,
+                                                                            const double *__restrict__ X, long long ldx,
+                                                                            const double *h, double *__restrict__ w,
+                                                                            double *part) {
+    pdl_enter();
+    double acc[PASS < 3 ? MM : 8];
+    __shared__ double hs[MM];
 #pragma unroll
-    for (int k = 0; k < MM; ++k) {
-        acc[k] = 0.0;
-        hk[k] = (PASS > 1 && k < m) ? h[k] : 0.0;
+    for (int k = 0; k < (PASS < 3 ? MM : 8); ++k) acc[k] = 0.0;
+    if (PASS > 1) {
+        if ((int)threadIdx.x < MM) hs[threadIdx.x] = (int)threadIdx.x < m ? h[threadIdx.x] : 0.0;
+        __syncthreads();
     }
+#pragma unroll(MM <= 8 ? 2 : 1)
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         double x[MM];
 #pragma unroll
@@ -341,7 +185,7 @@ __global__ void __launch_bounds__(RED_THREADS, MM <= 8 ? RED_BLOCKS / 152 : 1) k
         if (PASS > 1) {
 #pragma unroll
             for (int k = 0; k < MM; ++k)
-                if (k < m) v = fma(-hk[k], x[k], v);
+                if (k < m) v = fma(-hs[k], x[k], v);
             w[i] = v;
         }
         if (PASS < 3) {
@@ -352,37 +196,51 @@ __global__ void __launch_bounds__(RED_THREADS, MM <= 8 ? RED_BLOCKS / 152 : 1) k
             acc[0] = fma(v, v, acc[0]);
         }
     }
-    block_partials<MM>(acc, PASS < 3 ? m : 1, part);
+    block_partials<(PASS < 3 ? MM : 8)>(acc, PASS < 3 ? m : 1, part);
 }
 
 template <int MM>
-static void cgs_pass_mm(int pass, int n, int m, const double *X, long long ldx, const double *h, double *w, double *part,
-                        cudaStream_t s) {
-    if (pass == 1) k_cgs_pass<MM, 1><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, m, X, ldx, h, w, part);
-    else if (pass == 2) k_cgs_pass<MM, 2><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, m, X, ldx, h, w, part);
-    else k_cgs_pass<MM, 3><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, m, X, ldx, h, w, part);
+static void cgs_passes(int n, int m, const double *X, long long ldx, double *w, double *part, double *h1, double *h2,
+                       double *hsum, double *nrm, cudaStream_t s) {
+    int nb = red_blocks(n);
+    if (MM > 16 && nb > device_sms()) nb = device_sms();   // one block per SM is resident
+    launch_pdl(k_cgs_pass<MM, 1>, nb, RED_THREADS, 0, s, n, m, X, ldx, (const double *)nullptr, w, part);
+    finish(m, nb, part, h1, hsum, 1, s);
+    launch_pdl(k_cgs_pass<MM, 2>, nb, RED_THREADS, 0, s, n, m, X, ldx, (const double *)h1, w, part);
+    finish(m, nb, part, h2, hsum, 0, s);
+    launch_pdl(k_cgs_pass<MM, 3>, nb, RED_THREADS, 0, s, n, m, X, ldx, (const double *)h2, w, part);
+    finish(1, nb, part, nrm, nullptr, 1, s);
+    count_launch(3);
 }
 
-void cgs_pass(int pass, int n, int m, const double *X, long long ldx, const double *h, double *w, double *part,
-              cudaStream_t s) {
-    if (m <= 8) cgs_pass_mm<8>(pass, n, m, X, ldx, h, w, part, s);
-    else if (m <= 16) cgs_pass_mm<16>(pass, n, m, X, ldx, h, w, part, s);
-    else cgs_pass_mm<32>(pass, n, m, X, ldx, h, w, part, s);
-    count_launch();
+void cgs2(int n, int m, const double *X, long long ldx, double *w, double *part, double *h1, double *h2, double *hsum,
+          double *nrm, cudaStream_t s) {
+    if (m <= 8) cgs_passes<8>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, s);
+    else if (m <= 16) cgs_passes<16>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, s);
+    else if (m <= 24) cgs_passes<24>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, s);
+    else cgs_passes<32>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, s);
 }
 
-// v_out = v_in / *nrm (nrm = sqrt of a device scalar of squared norm)
-__global__ void k_scale_by_norm(int n, const double *__restrict__ v, const double *__restrict__ nrm2, double *__restrict__ out) {
+// v <- v / *nrm (nrm = sqrt of a device scalar of squared norm), and its copy c as the cycle's right-hand side
+template <class T>
+__global__ void k_scale_by_norm(int n, double *v, const double *nrm2, T *c) {
+    pdl_enter();
     const double n2 = *nrm2;
     const double inv = n2 > 0.0 ? 1.0 / sqrt(n2) : 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = v[i] * inv;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const double x = v[i] * inv;
+        v[i] = x;
+        c[i] = (T)x;
+    }
 }
 
-void scale_by_norm(int n, const double *v, const double *nrm2, double *out, cudaStream_t s) {
-    k_scale_by_norm<<<grid_for(n, 256, device_sms() * 8), 256, 0, s>>>(n, v, nrm2, out);
+template <class T>
+void scale_by_norm(int n, double *v, const double *nrm2, T *c, cudaStream_t s) {
+    launch_pdl(k_scale_by_norm<T>, grid_for(n, 256, device_sms() * 8), 256, 0, s, n, v, nrm2, c);
     count_launch();
 }
+template void scale_by_norm<float>(int, double *, const double *, float *, cudaStream_t);
+template void scale_by_norm<double>(int, double *, const double *, double *, cudaStream_t);
 
 // precision conversions and plain vector updates
 __global__ void k_d2f(int n, const double *__restrict__ a, float *__restrict__ b) {
@@ -484,7 +342,8 @@ __global__ void __launch_bounds__(256) k_tile_norm2(SegTiles st, const double *_
 // sum over the warps in order, as in k_tile_norm2.
 template <int MM, int PASS>
 __global__ void __launch_bounds__(256) k_tile_cgs(SegTiles st, int m, const double *__restrict__ X, long long ldx,
-                                                  int hs, const double *__restrict__ h, double *__restrict__ w) {
+                                                  int hs, const double *h, double *__restrict__ w) {
+    pdl_enter();
     __shared__ double red[8][MM];
     __shared__ double hsh[MM];
     for (int t = blockIdx.x; t < st.ntiles; t += gridDim.x) {
@@ -492,9 +351,9 @@ __global__ void __launch_bounds__(256) k_tile_cgs(SegTiles st, int m, const doub
         if (st.active && !st.active[tl.x]) continue;
         if (PASS > 1 && (int)threadIdx.x < MM) hsh[threadIdx.x] = (int)threadIdx.x < m ? h[(size_t)tl.x * hs + threadIdx.x] : 0.0;
         __syncthreads();
-        double acc[PASS < 3 ? MM : 1];
+        double acc[PASS < 3 ? MM : 8];
 #pragma unroll
-        for (int k = 0; k < (PASS < 3 ? MM : 1); ++k) acc[k] = 0.0;
+        for (int k = 0; k < (PASS < 3 ? MM : 8); ++k) acc[k] = 0.0;
         for (int i = tl.y + threadIdx.x; i < tl.z; i += blockDim.x) {
             double x[MM];
 #pragma unroll
@@ -508,7 +367,7 @@ __global__ void __launch_bounds__(256) k_tile_cgs(SegTiles st, int m, const doub
             }
             if (PASS < 3) {
 #pragma unroll
-                for (int k = 0; k < (PASS < 3 ? MM : 1); ++k)
+                for (int k = 0; k < (PASS < 3 ? MM : 8); ++k)
                     if (k < m) acc[k] = fma(x[k], v, acc[k]);
             } else {
                 acc[0] = fma(v, v, acc[0]);
@@ -516,10 +375,13 @@ __global__ void __launch_bounds__(256) k_tile_cgs(SegTiles st, int m, const doub
         }
         const int nout = PASS < 3 ? m : 1;
 #pragma unroll
-        for (int k = 0; k < (PASS < 3 ? MM : 1); ++k)
-            if (k < nout) {
-                const double v = warp_sum(acc[k]);
-                if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
+        for (int g = 0; g < (PASS < 3 ? MM : 8); g += 8)
+            if (g < nout) {
+                double u[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) u[k] = acc[g + k];
+                const double v = warp_sum8(u);
+                if ((threadIdx.x & 3) == 0) red[threadIdx.x >> 5][g + warp_sum8_index()] = v;
             }
         __syncthreads();
         if ((int)threadIdx.x < nout) {
@@ -531,21 +393,29 @@ __global__ void __launch_bounds__(256) k_tile_cgs(SegTiles st, int m, const doub
     }
 }
 
-// out[q * hs + k0 + k] = sum of the system's tile partials part[t * pw + k] in tile order (k < m);
-// acc_out[...] += the same when given. One warp per system.
-__global__ void __launch_bounds__(256) k_seg_reduce(SegTiles st, int pw, int m, int hs, int k0, double *__restrict__ out,
-                                                    double *__restrict__ acc_out) {
+// out[q * hs + k] = sum of the system's tile partials part[t * pw + k] (k < m): lane l adds tiles l, l + 32, ... and the
+// lanes' sums are added as a tree. acc_out (if any): = the same when first, else += it. One warp per system, eight
+// values at a time so that their loads overlap (one after another: 1,100 cycles each).
+__global__ void __launch_bounds__(256) k_seg_reduce(SegTiles st, int pw, int m, int hs, double *out, double *acc_out,
+                                                    int first) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < st.nseg; q += (gridDim.x * blockDim.x) >> 5) {
         if (st.active && !st.active[q]) continue;
         const int t0 = st.first[q], t1 = st.first[q + 1];
-        for (int k = 0; k < m; ++k) {
-            double v = 0.0;
-            for (int t = t0 + lane; t < t1; t += 32) v += st.part[(size_t)t * pw + k];
-            v = warp_sum(v);
-            if (lane == 0) {
-                out[(size_t)q * hs + k0 + k] = v;
-                if (acc_out) acc_out[(size_t)q * hs + k0 + k] += v;
+        for (int g = 0; g < m; g += 8) {
+            double v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = 0.0;
+            for (int t = t0 + lane; t < t1; t += 32)
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (g + k < m) v[k] += st.part[(size_t)t * pw + g + k];
+            const double r = warp_sum8(v);
+            const int k = g + warp_sum8_index();
+            if ((lane & 3) == 0 && k < m) {
+                out[(size_t)q * hs + k] = r;
+                if (acc_out) acc_out[(size_t)q * hs + k] = first ? r : acc_out[(size_t)q * hs + k] + r;
             }
         }
     }
@@ -569,14 +439,20 @@ __global__ void __launch_bounds__(256) k_tile_add_combo(SegTiles st, const int *
     }
 }
 
-__global__ void __launch_bounds__(256) k_tile_scale(SegTiles st, const double *__restrict__ v,
-                                                    const double *__restrict__ nrm2, double *__restrict__ out) {
+// v <- v / |v| per running system, and c = the same in T (the cycle's right-hand side)
+template <class T>
+__global__ void __launch_bounds__(256) k_tile_scale(SegTiles st, double *v, const double *nrm2, T *c) {
+    pdl_enter();
     for (int t = blockIdx.x; t < st.ntiles; t += gridDim.x) {
         const int4 tl = st.tile[t];
         if (st.active && !st.active[tl.x]) continue;
         const double n2 = nrm2[tl.x];
         const double inv = n2 > 0.0 ? 1.0 / sqrt(n2) : 0.0;
-        for (int i = tl.y + threadIdx.x; i < tl.z; i += blockDim.x) out[i] = v[i] * inv;
+        for (int i = tl.y + threadIdx.x; i < tl.z; i += blockDim.x) {
+            const double x = v[i] * inv;
+            v[i] = x;
+            c[i] = (T)x;
+        }
     }
 }
 
@@ -648,8 +524,9 @@ __global__ void k_bat_fg_restart(BatchCtl c, const double *__restrict__ nrm2, in
 // FGMRES step j of every running system: the new Hessenberg column (the Gram-Schmidt sums h[q * hs + k],
 // k <= j, and ||w||), the earlier rotations applied to it, a new rotation, the residual estimate and the
 // stopping test; a system that stops keeps its step count in jd
-__global__ void k_bat_fg_givens(BatchCtl c, int j, const double *__restrict__ hsum, const double *__restrict__ nrm2w,
+__global__ void k_bat_fg_givens(BatchCtl c, int j, const double *hsum, const double *nrm2w,
                                 int *count) {
+    pdl_enter();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= c.nseg || !c.run[q]) return;
     const int m = c.m;
@@ -708,7 +585,7 @@ void bat_fg_restart(const BatchCtl &c, const double *nrm2, int *count, cudaStrea
     count_launch();
 }
 void bat_fg_givens(const BatchCtl &c, int j, const double *hsum, const double *nrm2w, int *count, cudaStream_t s) {
-    k_bat_fg_givens<<<(c.nseg + 127) / 128, 128, 0, s>>>(c, j, hsum, nrm2w, count);
+    launch_pdl(k_bat_fg_givens, (c.nseg + 127) / 128, 128, 0, s, c, j, hsum, nrm2w, count);
     count_launch();
 }
 void bat_fg_solve_y(const BatchCtl &c, double *y, cudaStream_t s) {
@@ -718,17 +595,17 @@ void bat_fg_solve_y(const BatchCtl &c, double *y, cudaStream_t s) {
 
 static int seg_grid(const SegTiles &st) { return st.ntiles < SEG_GRID ? (st.ntiles > 0 ? st.ntiles : 1) : SEG_GRID; }
 
-static void seg_reduce(const SegTiles &st, int pw, int m, int hs, int k0, double *out, double *acc, cudaStream_t s) {
-    k_seg_reduce<<<(st.nseg + 7) / 8, 256, 0, s>>>(st, pw, m, hs, k0, out, acc);
+static void seg_reduce(const SegTiles &st, int pw, int m, int hs, double *out, double *acc, int first, cudaStream_t s) {
+    launch_pdl(k_seg_reduce, (st.nseg + 7) / 8, 256, 0, s, st, pw, m, hs, out, acc, first);
     count_launch();
 }
 
 template <int MM>
 static void seg_cgs_mm(const SegTiles &st, int pass, int m, const double *X, long long ldx, int hs, const double *h,
                        double *w, cudaStream_t s) {
-    if (pass == 1) k_tile_cgs<MM, 1><<<seg_grid(st), 256, 0, s>>>(st, m, X, ldx, hs, h, w);
-    else if (pass == 2) k_tile_cgs<MM, 2><<<seg_grid(st), 256, 0, s>>>(st, m, X, ldx, hs, h, w);
-    else k_tile_cgs<MM, 3><<<seg_grid(st), 256, 0, s>>>(st, m, X, ldx, hs, h, w);
+    if (pass == 1) launch_pdl(k_tile_cgs<MM, 1>, seg_grid(st), 256, 0, s, st, m, X, ldx, hs, h, w);
+    else if (pass == 2) launch_pdl(k_tile_cgs<MM, 2>, seg_grid(st), 256, 0, s, st, m, X, ldx, hs, h, w);
+    else launch_pdl(k_tile_cgs<MM, 3>, seg_grid(st), 256, 0, s, st, m, X, ldx, hs, h, w);
     count_launch();
 }
 
@@ -736,9 +613,10 @@ void seg_cgs_pass(const SegTiles &st, int pass, int m, const double *X, long lon
                   double *out, double *acc, cudaStream_t s) {
     if (m <= 8) seg_cgs_mm<8>(st, pass, m, X, ldx, hs, h, w, s);
     else if (m <= 16) seg_cgs_mm<16>(st, pass, m, X, ldx, hs, h, w, s);
+    else if (m <= 24) seg_cgs_mm<24>(st, pass, m, X, ldx, hs, h, w, s);
     else seg_cgs_mm<32>(st, pass, m, X, ldx, hs, h, w, s);
-    if (pass < 3) seg_reduce(st, SEG_TILE_PARTS, m, hs, 0, out, acc, s);
-    else seg_reduce(st, SEG_TILE_PARTS, 1, 1, 0, out, nullptr, s);
+    if (pass < 3) seg_reduce(st, SEG_TILE_PARTS, m, hs, out, acc, pass == 1, s);
+    else seg_reduce(st, SEG_TILE_PARTS, 1, 1, out, nullptr, 1, s);
 }
 
 void seg_add_combo(const SegTiles &st, const int *cnt, const double *Z, long long ldz, int hs, const double *y, double *x,
@@ -746,20 +624,23 @@ void seg_add_combo(const SegTiles &st, const int *cnt, const double *Z, long lon
     k_tile_add_combo<<<seg_grid(st), 256, 0, s>>>(st, cnt, Z, ldz, hs, y, x);
     count_launch();
 }
-void seg_scale(const SegTiles &st, const double *v, const double *nrm2, double *out, cudaStream_t s) {
-    k_tile_scale<<<seg_grid(st), 256, 0, s>>>(st, v, nrm2, out);
+template <class T>
+void seg_scale(const SegTiles &st, double *v, const double *nrm2, T *c, cudaStream_t s) {
+    launch_pdl(k_tile_scale<T>, seg_grid(st), 256, 0, s, st, v, nrm2, c);
     count_launch();
 }
+template void seg_scale<float>(const SegTiles &, double *, const double *, float *, cudaStream_t);
+template void seg_scale<double>(const SegTiles &, double *, const double *, double *, cudaStream_t);
 void seg_residual(const DCsr &A, const SegTiles &st, const double *b, const double *x, double *r, float *r32,
                   double *norm2, cudaStream_t s) {
     k_tile_residual<<<seg_grid(st), 256, 0, s>>>(st, A.rp, A.col, A.val, b, x, r, r32);
     count_launch();
-    seg_reduce(st, 1, 1, 1, 0, norm2, nullptr, s);
+    seg_reduce(st, 1, 1, 1, norm2, nullptr, 1, s);
 }
 void seg_norm2(const SegTiles &st, const double *v, double *norm2, cudaStream_t s) {
     k_tile_norm2<<<seg_grid(st), 256, 0, s>>>(st, v);
     count_launch();
-    seg_reduce(st, 1, 1, 1, 0, norm2, nullptr, s);
+    seg_reduce(st, 1, 1, 1, norm2, nullptr, 1, s);
 }
 template <class T>
 void seg_axpy(const SegTiles &st, const uint8_t *active, const T *e, double *x, cudaStream_t s) {
