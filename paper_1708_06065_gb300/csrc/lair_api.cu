@@ -471,15 +471,13 @@ static lair_status split_points(lair_handle *h, Temps &t, int l, int n, const Gr
         int2 *bd;
         TRY(t.get(&bd, blocks.size()));
         CU(cudaMemcpyAsync(bd, blocks.data(), sizeof(int2) * blocks.size(), cudaMemcpyHostToDevice, h->s));
-        // in-block entries of S, largest in-block row lengths of S and ST: they size the bucket queue
+        // in-block entries of S, largest in-block row lengths of S and ST: they choose the kernel and its shared memory
         int *mx, deg[3] = {0, 0, 0};
         TRY(new_counts(h, t, &mx, 3));
         launch_rs_degrees(bd, (int)blocks.size(), Scf, STcf, mx, h->s);
         TRY(read_ints(h, mx, 3, deg));   // also keeps the host block list alive until its copy is done
-        int nb = 8;
-        while (nb < 2 * deg[2] + 1) nb *= 2;
-        if (Bmax <= RSB_MAX_N && nb <= 256 && rsb_smem_bytes(Bmax, nb) <= (size_t)200 * 1024) {
-            CU(launch_rs_bucket(bd, (int)blocks.size(), Bmax, nb, deg[0], Scf, STcf, cf, h->status, h->s));
+        if (Bmax <= RSB_MAX_N && deg[2] <= RSB_MAX_DEG) {
+            CU(launch_rs_byte(bd, (int)blocks.size(), Bmax, deg[0], Scf, STcf, cf, h->status, h->s));
         } else {
             CU(launch_rs(n, bd, (int)blocks.size(), Bmax, deg[0], Scf, STcf, cf, h->status, h->s));
         }

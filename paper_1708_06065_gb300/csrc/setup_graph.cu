@@ -670,191 +670,148 @@ __global__ void __launch_bounds__(RS_DEG_THREADS) k_rs_degrees(const int2 *__res
 }
 
 // -------------------------------------------------------------------------------------
-// The same first pass with a bucket queue, for blocks of at most RSB_MAX_N points whose lambda
-// stays below nb buckets (lambda_k <= 2 |ST_k n block|: it starts at the in-block count and each
-// dependant adds one when it becomes F). Bucket b is a bitmap over the block of the undecided
-// points with lambda = b, so the point to take (largest lambda, then smallest index) is the lowest
-// set bit of the highest non-empty bucket. A step:
-//   1. find i, which becomes C;
-//   2. its undecided in-block dependants (ST_i) become F and leave their buckets;
+// The same first pass for blocks of at most RSB_MAX_N points whose lambda fits in a byte (lambda_k <= 2 |ST_k n block|:
+// it starts at the in-block count and each dependant adds one when it becomes F). Point k has one byte, lambda_k + 1,
+// or 0 once it is decided. Lane l of the warp that runs the steps keeps, in a register, the largest key of segment l
+// of the block, (lambda + 1) << 16 | (0xFFFF - index): largest lambda, then smallest index. A step:
+//   1. the largest of the lanes' keys names i, which becomes C;
+//   2. its undecided in-block dependants (ST_i) become F;
 //   3. lambda_k += 1 for undecided in-block k in S_j of every new F point j and lambda_k -= 1 for
-//      undecided in-block k in S_i; every such k moves to the bucket of its new lambda.
+//      undecided in-block k in S_i;
+//   4. the segments that hold a changed point are scanned again, by the whole warp.
 // The sequence of points taken is the one of the tree version above (and of the oracle).
 //
-// The steps depend on one another, so what bounds the kernel is the chain of shared-memory latencies of one
-// step. One warp runs them: the rows of step 3 (that of i and those of the new F points) are read four at a time
-// by eight lanes each, and the changes of one point that several lanes hold are summed with a warp match, so a
-// step is one pass of that chain however many neighbours it touches. (Walking S_j entry by entry in the lane
-// that made j an F point, with shared-memory atomics that return and a list of changed points: 1.4 us a step.)
-// The other warps of the CTA only help to set the block up.
+// The steps depend on one another, so what bounds the kernel is the chain of shared-memory latencies of one step. In
+// step 3 the rows (that of i and those of the new F points) are read four at a time by eight lanes each, and a change is
+// one shared-memory addition that returns nothing, so a step is one pass of that chain however many neighbours it
+// touches. 64^2 FD, 2,048 steps: 1.4 us a step with a lane walking S_j entry by entry through returning atomics and
+// bitmaps per lambda; 0.75 us with eight lanes per row and the changes of a point summed by a warp match (which takes
+// 377 cycles when the lanes hold different points); 0.58 us with this. The other warps of the CTA only help to set up.
 // -------------------------------------------------------------------------------------
 struct RsbLayout {
-    int W;                                // bitmap words per bucket (a multiple of 128)
-    size_t bm, cnt, lam, cf, total;       // byte offsets in dynamic shared memory
+    int shift;                            // 2^shift points per segment, at least 128
+    size_t cf, total;                     // byte offsets in dynamic shared memory (the keys come first)
 };
 
-__host__ __device__ inline size_t rsb_round16(size_t b) { return (b + 15) & ~(size_t)15; }
-
-__host__ __device__ inline RsbLayout rsb_layout(int n, int nb) {
+__host__ __device__ inline RsbLayout rsb_layout(int n) {
     RsbLayout L;
-    L.W = (((n + 31) / 32) + 127) / 128 * 128;
-    size_t o = 0;
-    L.bm = o;    o += rsb_round16((size_t)nb * L.W * sizeof(unsigned));
-    L.cnt = o;   o += rsb_round16((size_t)nb * sizeof(int));
-    L.lam = o;   o += rsb_round16((size_t)n);
-    L.cf = o;    o += rsb_round16((size_t)n);
-    L.total = o;
+    L.shift = 7;
+    while ((32 << L.shift) < n) ++L.shift;
+    L.cf = (size_t)32 << L.shift;
+    L.total = L.cf + (((size_t)n + 15) & ~(size_t)15);
     return L;
 }
 
 struct RsbShared {
-    unsigned *bm;      // nb bitmaps of W words
-    int *cnt;          // points per bucket
-    uint8_t *lam;      // lambda_k: the bucket that holds an undecided k
+    uint8_t *key;      // lambda + 1 of an undecided point, else 0; 32 segments
     int8_t *cf;
+    int shift;
 };
 
 // Step 3 for one set of rows: lane l holds the row [rb, re) of S (empty: no row) whose entries change by +1, or by -1
-// for the row of lane minus (the C point; -1: none). Returns the largest new lambda.
+// for the row of lane minus (the C point; -1: none). Returns this lane's mask of changed segments. A byte never leaves
+// 1 .. 255 on the way: k in S_i still counts i until it is taken off, and lambda_k <= 2 |ST_k| with it.
 template <class V>
-__device__ __forceinline__ int rsb_touch(int nb, int W, const V &Sv, const RsbShared &q, int rb, int re, int minus,
-                                         int *status) {
+__device__ __forceinline__ unsigned rsb_touch(const V &Sv, const RsbShared &q, int rb, int re, int minus) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    unsigned rows = __ballot_sync(FULL, rb < re);
-    int hi = 0;
-    while (rows) {
-        // the next four rows, eight lanes each
-        int src = -1;
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const int b = rows ? __ffs(rows) - 1 : -1;
-            if ((lane >> 3) == g) src = b;
-            rows &= rows - 1;   // 0 stays 0
-        }
-        int r = __shfl_sync(FULL, rb, src < 0 ? 0 : src) + (lane & 7);
-        const int e = __shfl_sync(FULL, re, src < 0 ? 0 : src);
-        const bool dec = src == minus;
-        bool in = src >= 0 && r < e;
+    const unsigned rows = __ballot_sync(FULL, rb < re);
+    unsigned dirty = 0;
+    for (int p = 0; rows >> p; p += 4) {   // four rows, eight lanes each
+        if (((rows >> p) & 15u) == 0) continue;
+        const int src = p + (lane >> 3);
+        int r = __shfl_sync(FULL, rb, src) + (lane & 7);
+        const int e = __shfl_sync(FULL, re, src);
         do {
-            int k = -1;
-            if (in) {
-                k = Sv.at(r);
-                if (k >= 0 && q.cf[k] != CF_U) k = -1;
-            }
-            // lanes that hold the same point: the lowest of them applies the sum of their changes
-            const unsigned same = __match_any_sync(FULL, k);
-            const unsigned down = __ballot_sync(FULL, dec);
-            if (k >= 0 && lane == __ffs(same) - 1) {
-                const int d = __popc(same & ~down) - __popc(same & down);
-                if (d != 0) {
-                    const int ob = q.lam[k], nl = ob + d;
-                    if (nl < 0 || nl >= nb) {   // the host sized nb above every reachable lambda
-                        set_status(status, LAIR_ERR_ARENA_OVERFLOW);
-                    } else {
-                        const unsigned bit = 1u << (k & 31);
-                        atomicAnd(&q.bm[ob * W + (k >> 5)], ~bit);
-                        atomicOr(&q.bm[nl * W + (k >> 5)], bit);
-                        atomicSub(&q.cnt[ob], 1);
-                        atomicAdd(&q.cnt[nl], 1);
-                        q.lam[k] = (uint8_t)nl;
-                        hi = max(hi, nl);
-                    }
+            if (r < e) {
+                const int k = Sv.at(r);
+                if (k >= 0 && q.key[k] != 0) {
+                    const unsigned one = 1u << (8 * (k & 3));
+                    atomicAdd(reinterpret_cast<unsigned *>(q.key) + (k >> 2), src == minus ? 0u - one : one);
+                    dirty |= 1u << (k >> q.shift);
                 }
             }
-            __syncwarp();
             r += 8;
-            in = src >= 0 && r < e;
-        } while (__any_sync(FULL, in));
+        } while (__any_sync(FULL, r < e));
+        __syncwarp();
     }
-    return hi;
+    return dirty;
 }
 
-// the steps of the bucket-queue first pass over in-block views of S and ST (local indices), one warp
+// the largest key of segment g, the same in every lane
+__device__ __forceinline__ unsigned rsb_scan(const RsbShared &q, int g) {
+    const int lane = threadIdx.x & 31;
+    unsigned m = 0;
+    for (int w0 = 0; w0 < 1 << q.shift; w0 += 128) {
+        const int at = (g << q.shift) + w0 + 4 * lane;
+        const unsigned w = *reinterpret_cast<const unsigned *>(q.key + at);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const unsigned k = (w >> (8 * b)) & 0xffu;
+            m = max(m, k ? (k << 16) | (0xFFFFu - (unsigned)(at + b)) : 0u);
+        }
+    }
+    return __reduce_max_sync(0xffffffffu, m);
+}
+
+// the steps of the first pass over in-block views of S and ST (local indices), one warp
 template <class V>
-__device__ void rsb_steps(int n, int nb, int W, int top, const V &Sv, const V &STv, const RsbShared &q, int *status) {
+__device__ void rsb_steps(int n, const V &Sv, const V &STv, const RsbShared &q) {
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
-    const int per = W / 32;                    // bitmap words scanned by each lane (4 or more, contiguous)
+    unsigned best = 0;
+    for (int g = 0; g < 32; ++g) {
+        const unsigned m = rsb_scan(q, g);
+        if (lane == g) best = m;
+    }
     for (int step = 0; step <= n; ++step) {
-        // 1. the highest non-empty bucket at or below top, then its lowest set bit
-        int b = -1;
-        for (int t0 = top; t0 >= 0; t0 -= 32) {
-            const int c = t0 - lane;
-            const unsigned m = __ballot_sync(FULL, c >= 0 && q.cnt[c] > 0);
-            if (m) {
-                b = t0 - (__ffs(m) - 1);
-                break;
-            }
-        }
-        if (b < 0) break;
-        top = b;
-        const unsigned *row = q.bm + (size_t)b * W + (size_t)lane * per;
-        int fw = -1;
-        unsigned fv = 0u;
-        for (int r = 0; r < per && fw < 0; r += 4) {
-            const uint4 u = *reinterpret_cast<const uint4 *>(row + r);
-            if (u.x) { fw = r; fv = u.x; }
-            else if (u.y) { fw = r + 1; fv = u.y; }
-            else if (u.z) { fw = r + 2; fv = u.z; }
-            else if (u.w) { fw = r + 3; fv = u.w; }
-        }
-        const unsigned fm = __ballot_sync(FULL, fw >= 0);
-        if (fm == 0u) {                        // a count without its bit: cannot happen
-            if (lane == 0) set_status(status, LAIR_ERR_DEVICE_TIMEOUT);
-            break;
-        }
-        const int src = __ffs(fm) - 1;
-        const int li = __shfl_sync(FULL, 32 * (fw + lane * per) + __ffs(fv) - 1, src);
-        // 2. li becomes C; its undecided in-block dependants become F (new in this step)
+        const unsigned top = __reduce_max_sync(FULL, best);
+        if (top == 0u) break;
+        const int li = (int)(0xFFFFu - (top & 0xFFFFu));
         const int sb = STv.beg(li), se = STv.end(li);
         const int ib = Sv.beg(li), ie = Sv.end(li);
         if (lane == 0) {
             q.cf[li] = CF_C;
-            atomicAnd(&q.bm[b * W + (li >> 5)], ~(1u << (li & 31)));
-            atomicSub(&q.cnt[b], 1);
+            q.key[li] = 0;
         }
-        auto leave = [&](int j) {
-            const int bj = q.lam[j];
-            atomicAnd(&q.bm[bj * W + (j >> 5)], ~(1u << (j & 31)));
-            atomicSub(&q.cnt[bj], 1);
-        };
-        int hi = 0;
+        unsigned dirty = 1u << (li >> q.shift);
         if (se - sb < 32) {
-            // lanes 0 .. 30: one dependant each; lane 31: the row of li itself
+            // lane 0: the row of li itself; the other lanes: one dependant each
             int rb = 0, re = 0;
-            if (lane < se - sb) {
-                const int j = STv.at(sb + lane);
+            if (lane == 0) {
+                rb = ib;
+                re = ie;
+            } else if (lane <= se - sb) {
+                const int j = STv.at(sb + lane - 1);
                 if (j >= 0) {
                     rb = Sv.beg(j);
                     re = Sv.end(j);
-                    if (q.cf[j] == CF_U) {
+                    if (q.key[j] != 0) {
                         q.cf[j] = CF_F;
-                        leave(j);
+                        q.key[j] = 0;
+                        dirty |= 1u << (j >> q.shift);
                     } else {
                         re = rb;
                     }
                 }
-            } else if (lane == 31) {
-                rb = ib;
-                re = ie;
             }
             __syncwarp();
-            hi = rsb_touch(nb, W, Sv, q, rb, re, 31, status);
+            dirty |= rsb_touch(Sv, q, rb, re, 0);
         } else {
             for (int p = sb + lane; p < se; p += 32) {
                 const int j = STv.at(p);
-                if (j >= 0 && q.cf[j] == CF_U) {
+                if (j >= 0 && q.key[j] != 0) {
                     q.cf[j] = CF_NEWF;
-                    leave(j);
+                    q.key[j] = 0;
+                    dirty |= 1u << (j >> q.shift);
                 }
             }
             __syncwarp();
-            hi = rsb_touch(nb, W, Sv, q, lane == 31 ? ib : 0, lane == 31 ? ie : 0, 31, status);
+            dirty |= rsb_touch(Sv, q, lane == 0 ? ib : 0, lane == 0 ? ie : 0, 0);
             for (int p0 = sb; p0 < se; p0 += 32) {
                 const int j = p0 + lane < se ? STv.at(p0 + lane) : -1;
                 const bool isnew = j >= 0 && q.cf[j] == CF_NEWF;
-                hi = max(hi, rsb_touch(nb, W, Sv, q, isnew ? Sv.beg(j) : 0, isnew ? Sv.end(j) : 0, -2, status));
+                dirty |= rsb_touch(Sv, q, isnew ? Sv.beg(j) : 0, isnew ? Sv.end(j) : 0, -1);
             }
             for (int p = sb + lane; p < se; p += 32) {
                 const int j = STv.at(p);
@@ -862,7 +819,13 @@ __device__ void rsb_steps(int n, int nb, int W, int top, const V &Sv, const V &S
             }
             __syncwarp();
         }
-        top = max(top, (int)__reduce_max_sync(FULL, (unsigned)hi));
+        dirty = __reduce_or_sync(FULL, dirty);
+        while (dirty) {
+            const int g = __ffs(dirty) - 1;
+            dirty &= dirty - 1;
+            const unsigned m = rsb_scan(q, g);
+            if (lane == g) best = m;
+        }
     }
 }
 
@@ -918,49 +881,37 @@ __device__ bool rsb_stage(const Graph &G, int b0, int b1, uint16_t *rp, uint16_t
     return true;
 }
 
-// smem_bytes: the bucket layout of the largest block, plus (stage != 0) room to stage both in-block graphs
+// smem_bytes: the layout of the largest block, plus (stage != 0) room to stage both in-block graphs
 // (uint16 row offsets and columns) so that each step reads shared memory only. Staging pays when the level
 // has at most one block per SM; with more blocks it costs occupancy, which hides more of each step's
 // latency than the staging saves (measured), and the graphs are read through the cache.
-__global__ void __launch_bounds__(RSB_THREADS) k_rs_bucket(const int2 *__restrict__ blocks, Graph S, Graph ST, int nb,
-                                                           int8_t *__restrict__ cf_out, int *status, int stage,
-                                                           int smem_bytes) {
+__global__ void __launch_bounds__(RSB_THREADS) k_rs_byte(const int2 *__restrict__ blocks, Graph S, Graph ST,
+                                                         int8_t *__restrict__ cf_out, int *status, int stage,
+                                                         int smem_bytes) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int top_s;
     const int b0 = blocks[blockIdx.x].x, b1 = blocks[blockIdx.x].y;
     const int n = b1 - b0, t = threadIdx.x, T = blockDim.x;
-    const RsbLayout Lo = rsb_layout(n, nb);
-    const int W = Lo.W;
+    const RsbLayout Lo = rsb_layout(n);
     RsbShared q;
-    q.bm = reinterpret_cast<unsigned *>(smem + Lo.bm);
-    q.cnt = reinterpret_cast<int *>(smem + Lo.cnt);
-    q.lam = smem + Lo.lam;
+    q.key = smem;
     q.cf = reinterpret_cast<int8_t *>(smem + Lo.cf);
-
-    for (int e = t; e < nb * W; e += T) q.bm[e] = 0u;
-    for (int e = t; e < nb; e += T) q.cnt[e] = 0;
-    if (t == 0) top_s = 0;
-    __syncthreads();
-    int top = 0;
-    for (int li = t; li < n; li += T) {
+    q.shift = Lo.shift;
+    for (int li = t; li < 32 << Lo.shift; li += T) {
+        if (li >= n) {
+            q.key[li] = 0;
+            continue;
+        }
         const int i = b0 + li;
         int lam = 0;
         for (int p = ST.rp[i]; p < ST.rp[i + 1]; ++p) lam += (ST.col[p] >= b0 && ST.col[p] < b1);
         const bool iso = (S.rp[i + 1] == S.rp[i]) && (ST.rp[i + 1] == ST.rp[i]);
-        q.cf[li] = iso ? CF_F : CF_U;
-        q.lam[li] = 0;
-        if (iso) continue;
-        if (lam >= nb) {                       // the host sized nb above every reachable lambda
+        if (lam > 254) {                       // the host has seen to it that every reachable lambda fits
             set_status(status, LAIR_ERR_ARENA_OVERFLOW);
-            lam = nb - 1;
+            lam = 254;
         }
-        q.lam[li] = (uint8_t)lam;
-        atomicOr(&q.bm[lam * W + (li >> 5)], 1u << (li & 31));
-        atomicAdd(&q.cnt[lam], 1);
-        top = max(top, lam);
+        q.cf[li] = iso ? CF_F : CF_U;
+        q.key[li] = iso ? (uint8_t)0 : (uint8_t)(lam + 1);
     }
-    top = (int)__reduce_max_sync(0xffffffffu, (unsigned)top);
-    if ((t & 31) == 0) atomicMax(&top_s, top);
     __syncthreads();
     bool staged = false;
     uint16_t *srp = reinterpret_cast<uint16_t *>(smem + Lo.total);
@@ -973,13 +924,12 @@ __global__ void __launch_bounds__(RSB_THREADS) k_rs_bucket(const int2 *__restric
         if (staged) staged = rsb_stage(ST, b0, b1, strp, scol + srp[n], cap);
     }
     if (t < 32) {
-        top = top_s;
         if (staged) {
             StagedView vs{srp, scol}, vt{strp, scol + srp[n]};
-            rsb_steps(n, nb, W, top, vs, vt, q, status);
+            rsb_steps(n, vs, vt, q);
         } else {
             GlobalView vs{S.rp, S.col, b0, b1}, vt{ST.rp, ST.col, b0, b1};
-            rsb_steps(n, nb, W, top, vs, vt, q, status);
+            rsb_steps(n, vs, vt, q);
         }
     }
     __syncthreads();
@@ -989,8 +939,6 @@ __global__ void __launch_bounds__(RSB_THREADS) k_rs_bucket(const int2 *__restric
         cf_out[b0 + li] = c;
     }
 }
-
-size_t rsb_smem_bytes(int n, int nb) { return rsb_layout(n, nb).total; }
 
 // the bytes to stage both in-block graphs of the fullest block as well
 static size_t rsb_stage_bytes(int n, int max_inblock) {
@@ -1359,20 +1307,20 @@ void launch_rs_degrees(const int2 *blocks, int nblocks, const Graph &S, const Gr
     count_launch();
 }
 
-cudaError_t launch_rs_bucket(const int2 *blocks, int nblocks, int Bmax, int nb, int max_inblock, const Graph &S,
-                             const Graph &ST, int8_t *cf, int *status, cudaStream_t s) {
-    size_t bytes = rsb_smem_bytes(Bmax, nb);
+cudaError_t launch_rs_byte(const int2 *blocks, int nblocks, int Bmax, int max_inblock, const Graph &S, const Graph &ST,
+                           int8_t *cf, int *status, cudaStream_t s) {
+    size_t bytes = rsb_layout(Bmax).total;
     int stage = 0;
     if (nblocks <= device_sms()) {
         const size_t want = bytes + rsb_stage_bytes(Bmax, max_inblock);
         stage = 1;
         bytes = want < (size_t)RS_SMEM_MAX ? want : (bytes > (size_t)RS_SMEM_MAX ? bytes : (size_t)RS_SMEM_MAX);
     }
-    cudaError_t e = cudaFuncSetAttribute(k_rs_bucket, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = cudaFuncSetAttribute(k_rs_byte, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     // a few warps to set the block up; many blocks on an SM need no more than two each
     const int tb = stage ? RSB_THREADS : 64;
-    k_rs_bucket<<<nblocks, tb, bytes, s>>>(blocks, S, ST, nb, cf, status, stage, (int)bytes);
+    k_rs_byte<<<nblocks, tb, bytes, s>>>(blocks, S, ST, cf, status, stage, (int)bytes);
     count_launch();
     return cudaGetLastError();
 }

@@ -50,15 +50,15 @@ constexpr long long GRID_WAIT_POLLS = 1ll << 22;
 cudaError_t launch_pmis_all(int n, const Graph &S, const Graph &ST, double *w, int8_t *cf, int8_t *newc, int *lists,
                             int *ctl, int *status, int wait_polls, cudaStream_t s);
 void launch_rs_count(const int2 *blocks, int nblocks, const Graph &S, int *maxcnt, cudaStream_t s);
-// bucket-queue first pass: blocks of at most RSB_MAX_N points, lambda below nb <= 256 buckets
+// first pass with a byte per point: blocks of at most RSB_MAX_N points with at most RSB_MAX_DEG in-block dependants each
 constexpr int RSB_MAX_N = 8192;
+constexpr int RSB_MAX_DEG = 127;   // lambda + 1 <= 2 * 127 + 1
 constexpr int RSB_THREADS = 256;
 void launch_rs_degrees(const int2 *blocks, int nblocks, const Graph &S, const Graph &ST, int *out, cudaStream_t s);
 // (levels of at most one block per SM stage the in-block graphs in shared memory; max_inblock: the largest
 // in-block entry count of S)
-cudaError_t launch_rs_bucket(const int2 *blocks, int nblocks, int Bmax, int nb, int max_inblock,
-                             const Graph &S, const Graph &ST, int8_t *cf, int *status, cudaStream_t s);
-size_t rsb_smem_bytes(int n, int nb);
+cudaError_t launch_rs_byte(const int2 *blocks, int nblocks, int Bmax, int max_inblock, const Graph &S, const Graph &ST,
+                           int8_t *cf, int *status, cudaStream_t s);
 cudaError_t launch_rs(int n, const int2 *blocks, int nblocks, int Bmax, int max_inblock, const Graph &S, const Graph &ST,
                       int8_t *cf, int *status, cudaStream_t s);
 size_t rs_smem_bytes(int n, int max_inblock);

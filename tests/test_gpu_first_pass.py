@@ -1,4 +1,4 @@
-"""The bucket-queue first pass against the oracle where one of its paths ends: rows of ST with 31, 32 and more
+"""The first pass against the oracle where one of its paths ends: rows of ST with 31, 32 and more than 127
 dependants, rows of S longer than the eight lanes that share one, several blocks (staged graphs, and more blocks than
 SMs, read through the cache), points without any strong connection."""
 import numpy as np
@@ -50,6 +50,7 @@ def star(hubs, leaves):
 SYSTEMS = {
     "star30": lambda: star(9, 30), "star31": lambda: star(9, 31), "star32": lambda: star(7, 32),
     "star33": lambda: star(7, 33), "star100": lambda: star(5, 100),
+    "star126": lambda: star(3, 126), "star127": lambda: star(3, 127), "star140": lambda: star(3, 140),
     "random": lambda: W.random_sparse(3000, 12, 4, sym_pattern=True), "wide": lambda: W.random_sparse(700, 40, 5),
     "fd2d": lambda: W.fd_adr_2d(90, 0.4, 1e-2, 0.1), "fd3d": lambda: W.fd_adr_3d(22, (1.0, 0.7, 0.4), 1e-3, 0.1),
     "chain": lambda: W.upwind_chain(257),
