@@ -84,7 +84,7 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
             int tr = tbegin(h, "outer_residual", (double)A.nnz * 12.0 + (double)n * (4.0 + 16.0 + (mixed ? 4.0 : 8.0)));
             sell_residual(L0.A64, b, x, mixed ? nullptr : L0.b64, mixed ? L0.b32 : nullptr, h->part, h->s);
             tend(h, tr);
-            finish_residual(h->part, h->dsc, h->s);
+            finish_residual(h->part, h->dsc, nullptr, h->s);
             CU(cudaMemcpyAsync(h->h_dbl, h->dsc, sizeof(double), cudaMemcpyDeviceToHost, h->s));
             CU(cudaStreamSynchronize(h->s));
 
@@ -107,13 +107,14 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
         // device scalars: |r|^2 or |w|^2 at 7, Hessenberg column behind it (32), the two CGS2 projections at 48 (64), y
         // at 112 (32)
         double *nrm = h->dsc + 7, *hsum = nrm + 1, *hbuf = h->dsc + 48, *ydev = h->dsc + 112;
-        auto scale = [&](double *v) {   // v <- v / |v|, also into the cycle's right-hand side
-            if (mixed) scale_by_norm<float>(n, v, nrm, L0.b32, h->s);
-            else scale_by_norm<double>(n, v, nrm, L0.b64, h->s);
+        double *inv = h->dsc + 6;       // the inverse of the norm at 7's root
+        auto unit = [&](double *v) {   // v <- v / |v|, also into the cycle's right-hand side
+            if (mixed) scale<float>(n, v, inv, L0.b32, h->s);
+            else scale<double>(n, v, inv, L0.b64, h->s);
         };
         if (!h->col_ev) CU(cudaEventCreateWithFlags(&h->col_ev, cudaEventDisableTiming));
         sell_residual(L0.A64, b, x, V, nullptr, h->part, h->s);
-        finish_residual(h->part, nrm, h->s);
+        finish_residual(h->part, nrm, inv, h->s);
         CU(cudaMemcpyAsync(h->h_dbl, nrm, sizeof(double), cudaMemcpyDeviceToHost, h->s));
         CU(cudaStreamSynchronize(h->s));
 
@@ -122,7 +123,7 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
         rel = beta / bn;
         hist(rel);
         while (std::isfinite(rel) && rel > tol && it < max_iter) {
-            scale(V);
+            unit(V);
             std::fill(g.begin(), g.end(), 0.0);
             g[0] = beta;
             int jdone = 0;
@@ -135,11 +136,11 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
                 else sell_spmv_keep<double>(L0.A64, L0.x64[L0.xfinal], zj, w, h->s);
                 tend(h, ts);
                 int to = tbegin(h, "outer_cgs2", 8.0 * n * (3.0 * (j + 2) + 4.0));
-                cgs2(n, j + 1, V, n, w, h->part, hbuf, hbuf + 32, hsum, nrm, h->s);
+                cgs2(n, j + 1, V, n, w, h->part, hbuf, hbuf + 32, hsum, nrm, inv, h->s);
                 // the host reads the column and goes on while w is being scaled
                 CU(cudaMemcpyAsync(h->h_dbl, nrm, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, h->s));
                 CU(cudaEventRecord(h->col_ev, h->s));
-                scale(w);
+                unit(w);
                 tend(h, to);
                 if (h->o.timing) {
                     CU(cudaStreamSynchronize(h->s));
@@ -175,7 +176,7 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
             CU(cudaMemcpyAsync(ydev, y.data(), sizeof(double) * jdone, cudaMemcpyHostToDevice, h->s));
             add_combo(n, jdone, Z, n, ydev, x, h->s);
             sell_residual(L0.A64, b, x, V, nullptr, h->part, h->s);
-            finish_residual(h->part, nrm, h->s);
+            finish_residual(h->part, nrm, inv, h->s);
             CU(cudaMemcpyAsync(h->h_dbl, nrm, sizeof(double), cudaMemcpyDeviceToHost, h->s));
             CU(cudaStreamSynchronize(h->s));
 

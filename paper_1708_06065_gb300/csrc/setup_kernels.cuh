@@ -191,15 +191,16 @@ constexpr int RED_PARTS = 152 * 4;
 // r = b - A x over an FP64 sliced-ELL view of all rows (r and its FP32 copy optional); |r|^2 as RED_PARTS block partials
 void sell_residual(const SellView &v, const double *b, const double *x, double *r, float *r32, double *part,
                    cudaStream_t s);
-void finish_residual(const double *part, double *out, cudaStream_t s);   // the sum of sell_residual's partials
+// the sum of sell_residual's partials; inv (may be NULL): 1 / sqrt of it, 0 for 0
+void finish_residual(const double *part, double *out, double *inv, cudaStream_t s);
 void norm2(int n, const double *v, double *part, double *out, cudaStream_t s);
-// CGS2 of w against the m <= 32 columns of X: the sums of both projections to hsum, the new |w|^2 to nrm; part, h1 and
+// CGS2 of w against the m <= 32 columns of X: the sums of both projections to hsum, the new |w|^2 to nrm, 1 / |w| to inv; part, h1 and
 // h2 (32 each): scratch
 void cgs2(int n, int m, const double *X, long long ldx, double *w, double *part, double *h1, double *h2, double *hsum,
-          double *nrm, cudaStream_t s);
+          double *nrm, double *inv, cudaStream_t s);
 void add_combo(int n, int m, const double *Z, long long ldz, const double *y, double *x, cudaStream_t s);
-// v <- v / sqrt(*nrm2), and c = the same in T
-template <class T> void scale_by_norm(int n, double *v, const double *nrm2, T *c, cudaStream_t s);
+// v <- v * *inv, and c = the same in T
+template <class T> void scale(int n, double *v, const double *inv, T *c, cudaStream_t s);
 void d2f(int n, const double *a, float *b, cudaStream_t s);
 void f2d(int n, const float *a, double *b, cudaStream_t s);
 void axpy_f(int n, const float *e, double *x, cudaStream_t s);

@@ -87,8 +87,10 @@ static int red_blocks(int n) {
     return g < RED_PARTS ? g : RED_PARTS;
 }
 
-// out[k] = sum of the nb partials of vector k (fixed order); acc (if any): acc[k] = out[k] when first, else += out[k]
-__global__ void __launch_bounds__(128) k_finish(int m, int nb, const double *part, double *out, double *acc, int first) {
+// out[k] = sum of the nb partials of vector k (fixed order); acc (if any): acc[k] = out[k] when first, else += out[k];
+// inv (if any): 1 / sqrt(out[0]), 0 for a zero vector
+__global__ void __launch_bounds__(128) k_finish(int m, int nb, const double *part, double *out, double *acc, int first,
+                                                double *inv) {
     pdl_enter();
     const int k = blockIdx.x;
     if (k >= m) return;
@@ -102,16 +104,18 @@ __global__ void __launch_bounds__(128) k_finish(int m, int nb, const double *par
         const double u = ((red[0] + red[1]) + red[2]) + red[3];
         out[k] = u;
         if (acc) acc[k] = first ? u : acc[k] + u;
+        if (inv && k == 0) *inv = u > 0.0 ? 1.0 / sqrt(u) : 0.0;
     }
 }
 
-static void finish(int m, int nb, const double *part, double *out, double *acc, int first, cudaStream_t s) {
-    launch_pdl(k_finish, m, 128, 0, s, m, nb, part, out, acc, first);
+static void finish(int m, int nb, const double *part, double *out, double *acc, int first, cudaStream_t s,
+                   double *inv = nullptr) {
+    launch_pdl(k_finish, m, 128, 0, s, m, nb, part, out, acc, first, inv);
     count_launch();
 }
 
-void finish_residual(const double *part, double *out, cudaStream_t s) {
-    finish(1, RED_PARTS, part, out, nullptr, 1, s);
+void finish_residual(const double *part, double *out, double *inv, cudaStream_t s) {
+    finish(1, RED_PARTS, part, out, nullptr, 1, s, inv);
 }
 
 // |v|^2 as block partials
@@ -201,7 +205,7 @@ __global__ void __launch_bounds__(RED_THREADS, MM <= 16 ? 2 : 1) k_cgs_pass(int 
 
 template <int MM>
 static void cgs_passes(int n, int m, const double *X, long long ldx, double *w, double *part, double *h1, double *h2,
-                       double *hsum, double *nrm, cudaStream_t s) {
+                       double *hsum, double *nrm, double *inv, cudaStream_t s) {
     int nb = red_blocks(n);
     if (MM > 16 && nb > device_sms()) nb = device_sms();   // one block per SM is resident
     launch_pdl(k_cgs_pass<MM, 1>, nb, RED_THREADS, 0, s, n, m, X, ldx, (const double *)nullptr, w, part);
@@ -209,38 +213,51 @@ static void cgs_passes(int n, int m, const double *X, long long ldx, double *w, 
     launch_pdl(k_cgs_pass<MM, 2>, nb, RED_THREADS, 0, s, n, m, X, ldx, (const double *)h1, w, part);
     finish(m, nb, part, h2, hsum, 0, s);
     launch_pdl(k_cgs_pass<MM, 3>, nb, RED_THREADS, 0, s, n, m, X, ldx, (const double *)h2, w, part);
-    finish(1, nb, part, nrm, nullptr, 1, s);
+    finish(1, nb, part, nrm, nullptr, 1, s, inv);
     count_launch(3);
 }
 
 void cgs2(int n, int m, const double *X, long long ldx, double *w, double *part, double *h1, double *h2, double *hsum,
-          double *nrm, cudaStream_t s) {
-    if (m <= 8) cgs_passes<8>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, s);
-    else if (m <= 16) cgs_passes<16>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, s);
-    else if (m <= 24) cgs_passes<24>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, s);
-    else cgs_passes<32>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, s);
+          double *nrm, double *inv, cudaStream_t s) {
+    if (m <= 8) cgs_passes<8>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, inv, s);
+    else if (m <= 16) cgs_passes<16>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, inv, s);
+    else if (m <= 24) cgs_passes<24>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, inv, s);
+    else cgs_passes<32>(n, m, X, ldx, w, part, h1, h2, hsum, nrm, inv, s);
 }
 
-// v <- v / *nrm (nrm = sqrt of a device scalar of squared norm), and its copy c as the cycle's right-hand side
+// v <- v * *inv, and its copy c as the cycle's right-hand side. The inverse norm comes from the kernel that summed the
+// norm: formed here by every thread, its root and division cost the FP64 units more than the whole vector costs HBM
+// (101^3: 14.1 us -> 6.5).
 template <class T>
-__global__ void k_scale_by_norm(int n, double *v, const double *nrm2, T *c) {
+__global__ void __launch_bounds__(256) k_scale(int n, double *__restrict__ v, const double *inv, T *__restrict__ c) {
     pdl_enter();
-    const double n2 = *nrm2;
-    const double inv = n2 > 0.0 ? 1.0 / sqrt(n2) : 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const double x = v[i] * inv;
+    const double f = *inv;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (; i + 3 * stride < n; i += 4 * stride) {
+        double x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = v[i + k * stride] * f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[i + k * stride] = x[k];
+            c[i + k * stride] = (T)x[k];
+        }
+    }
+    for (; i < n; i += stride) {
+        const double x = v[i] * f;
         v[i] = x;
         c[i] = (T)x;
     }
 }
 
 template <class T>
-void scale_by_norm(int n, double *v, const double *nrm2, T *c, cudaStream_t s) {
-    launch_pdl(k_scale_by_norm<T>, grid_for(n, 256, device_sms() * 8), 256, 0, s, n, v, nrm2, c);
+void scale(int n, double *v, const double *inv, T *c, cudaStream_t s) {
+    launch_pdl(k_scale<T>, grid_for(n, 256, device_sms() * 8), 256, 0, s, n, v, inv, c);
     count_launch();
 }
-template void scale_by_norm<float>(int, double *, const double *, float *, cudaStream_t);
-template void scale_by_norm<double>(int, double *, const double *, double *, cudaStream_t);
+template void scale<float>(int, double *, const double *, float *, cudaStream_t);
+template void scale<double>(int, double *, const double *, double *, cudaStream_t);
 
 // precision conversions and plain vector updates
 __global__ void k_d2f(int n, const double *__restrict__ a, float *__restrict__ b) {
@@ -251,19 +268,25 @@ __global__ void k_f2d(int n, const float *__restrict__ a, double *__restrict__ b
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         b[i] = (double)a[i];
 }
-__global__ void k_axpy_f(int n, const float *__restrict__ e, double *__restrict__ x) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        x[i] += (double)e[i];
-}
-__global__ void k_axpy_d(int n, const double *__restrict__ e, double *__restrict__ x) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        x[i] += e[i];
+// x += e, four elements of a thread in flight (bound by HBM; 192^3: 34.7 us with one -> 31.8)
+template <class T>
+__global__ void __launch_bounds__(256) k_axpy(int n, const T *__restrict__ e, double *__restrict__ x) {
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (; i + 3 * stride < n; i += 4 * stride) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = x[i + k * stride] + (double)e[i + k * stride];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[i + k * stride] = v[k];
+    }
+    for (; i < n; i += stride) x[i] += (double)e[i];
 }
 
 void d2f(int n, const double *a, float *b, cudaStream_t s) { k_d2f<<<grid_for(n, 256, device_sms() * 8), 256, 0, s>>>(n, a, b); count_launch(); }
 void f2d(int n, const float *a, double *b, cudaStream_t s) { k_f2d<<<grid_for(n, 256, device_sms() * 8), 256, 0, s>>>(n, a, b); count_launch(); }
-void axpy_f(int n, const float *e, double *x, cudaStream_t s) { k_axpy_f<<<grid_for(n, 256, device_sms() * 8), 256, 0, s>>>(n, e, x); count_launch(); }
-void axpy_d(int n, const double *e, double *x, cudaStream_t s) { k_axpy_d<<<grid_for(n, 256, device_sms() * 8), 256, 0, s>>>(n, e, x); count_launch(); }
+void axpy_f(int n, const float *e, double *x, cudaStream_t s) { k_axpy<float><<<grid_for(n, 256, device_sms() * 8), 256, 0, s>>>(n, e, x); count_launch(); }
+void axpy_d(int n, const double *e, double *x, cudaStream_t s) { k_axpy<double><<<grid_for(n, 256, device_sms() * 8), 256, 0, s>>>(n, e, x); count_launch(); }
 
 // adjoint gradient on the pattern of A: g[k] = -lambda_i x_j
 __global__ void k_grad_A(int n, const int *__restrict__ rp, const int *__restrict__ col, const double *__restrict__ lam,
@@ -443,11 +466,14 @@ __global__ void __launch_bounds__(256) k_tile_add_combo(SegTiles st, const int *
 template <class T>
 __global__ void __launch_bounds__(256) k_tile_scale(SegTiles st, double *v, const double *nrm2, T *c) {
     pdl_enter();
+    __shared__ double inv_s;   // one thread's root and division for the tile: they are what the FP64 units cost
     for (int t = blockIdx.x; t < st.ntiles; t += gridDim.x) {
         const int4 tl = st.tile[t];
         if (st.active && !st.active[tl.x]) continue;
-        const double n2 = nrm2[tl.x];
-        const double inv = n2 > 0.0 ? 1.0 / sqrt(n2) : 0.0;
+        __syncthreads();
+        if (threadIdx.x == 0) inv_s = nrm2[tl.x] > 0.0 ? 1.0 / sqrt(nrm2[tl.x]) : 0.0;
+        __syncthreads();
+        const double inv = inv_s;
         for (int i = tl.y + threadIdx.x; i < tl.z; i += blockDim.x) {
             const double x = v[i] * inv;
             v[i] = x;
