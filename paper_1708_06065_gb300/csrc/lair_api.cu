@@ -269,8 +269,10 @@ static lair_status local_rows(lair_handle *h, Temps &t, int nc, const int *cpts,
     TRY(new_counts(h, t, &ub, nc));
     launch_nb_bound(nc, cpts, G, cf, d0, ub, h->s);
     TRY(t.get(&off, (size_t)nc + 1));
-    int total = 0;
-    TRY(scan(h, ub, off, nc, &total));
+    // at distance one a set is part of the point's row of G, so G's capacity bounds their total; beyond, it is read back
+    // (12 us in which the GPU waits for the host)
+    int total = G.nnz;
+    TRY(scan(h, ub, off, nc, d0 == 1 ? nullptr : &total));
     TRY(t.get(&tmp, (size_t)total));
     TRY(new_counts(h, t, &cnt, nc));
     launch_nb_fill(nc, cpts, G, cf, d0, off, tmp, cnt, h->s);
