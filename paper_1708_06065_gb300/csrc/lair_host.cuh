@@ -52,6 +52,8 @@ struct Level {
     int *frows = nullptr, *crows = nullptr;
     SellView AF, AC, Rv, Pv;
     SellView A64;             // level 0: all rows of A in FP64 for the outer iteration
+    bool split = false;       // the F sweeps do not copy the C rows: P writes them to both x buffers; below level 0 the C
+                              // sweep does not copy the F rows either, and the result is F points in x[0], C in x[1]
     int *p1col = nullptr;     // one-point P (every entry 1): the coarse column of each row's entry, -1 without one
     int *blk_sys = nullptr;   // batched systems: the system of every 32-row block of the level (-1: several)
     // nodal hierarchy (k x k blocks): block Jacobi as point Jacobi on Ahat = D^{-1} A (diagonal blocks

@@ -454,24 +454,37 @@ __global__ void __launch_bounds__(WAVE_THREADS) k_sell_sweep_wave(SellView v, co
 // row, every entry 1): x_i = x_c[col_i] + 0, or 0 for a row without an entry -- the bits of fma(1, x_c[col_i], 0)
 // that the sliced-ELL product gives (a -0 becomes +0). One column per row from the dense column array, one
 // gather, one write: coalesced everywhere but the gather.
+//
+// Two flags above the column (P1_MASK) spare the sweeps their copies of the rows they do not touch (split_p1_cols):
+// P1_SECOND: the coarse point is a C point of a level whose result lies in two vectors, F points in the first and C
+// points in the second; P1_BOTH: the row is a C point, written to x and x2, so that the F sweeps can go from one to the
+// other without carrying the C points along.
 template <class T>
-__global__ void __launch_bounds__(256) k_p1_interp(int n, const int *__restrict__ p1col, const int *__restrict__ blk_sys,
-                                                   const uint8_t *run, const T *__restrict__ xc, T *__restrict__ x) {
+__device__ __forceinline__ void p1_row(int c, int mask, const T *xc, const T *xc2, T *x, T *x2, int i) {
+    const T v = c >= 0 ? ((c & ~mask & P1_SECOND) ? xc2 : xc)[c & mask] + T(0) : T(0);
+    x[i] = v;
+    if (c >= 0 && (c & ~mask & P1_BOTH)) x2[i] = v;
+}
+
+template <class T>
+__global__ void __launch_bounds__(256) k_p1_interp(int n, const int *__restrict__ p1col, int mask,
+                                                   const int *__restrict__ blk_sys, const uint8_t *run,
+                                                   const T *__restrict__ xc, const T *__restrict__ xc2,
+                                                   T *__restrict__ x, T *__restrict__ x2) {
     pdl_enter();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         if (run) {
             const int q = blk_sys[i >> 5];
             if (q >= 0 && !run[q]) continue;
         }
-        const int c = __ldcs(p1col + i);
-        x[i] = c >= 0 ? __ldg(xc + c) + T(0) : T(0);
+        p1_row<T>(__ldcs(p1col + i), mask, xc, xc2, x, x2, i);
     }
 }
 
 // the same in one wave, a row per thread: the column is read before the previous kernel has finished
 template <class T>
-__global__ void __launch_bounds__(256) k_p1_interp_wave(int n, const int *p1col, const int *blk_sys, const uint8_t *run,
-                                                        const T *xc, T *x) {
+__global__ void __launch_bounds__(256) k_p1_interp_wave(int n, const int *p1col, int mask, const int *blk_sys,
+                                                        const uint8_t *run, const T *xc, const T *xc2, T *x, T *x2) {
     pdl_launch_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     bool on = i < n;
@@ -481,19 +494,43 @@ __global__ void __launch_bounds__(256) k_p1_interp_wave(int n, const int *p1col,
     }
     const int c = on ? __ldg(p1col + i) : -1;
     pdl_wait_previous();
-    if (on) x[i] = c >= 0 ? xc[c] + T(0) : T(0);
+    if (on) p1_row<T>(c, mask, xc, xc2, x, x2, i);
 }
 
 template <class T>
-void p1_interp(int n, const int *p1col, const int *blk_sys, const uint8_t *run, const T *xc, T *x, cudaStream_t s) {
+void p1_interp(int n, const int *p1col, bool flags, const int *blk_sys, const uint8_t *run, const T *xc, const T *xc2,
+               T *x, T *x2, cudaStream_t s) {
     if (n <= 0) return;
-    if (n <= one_wave_rows<T>()) launch_pdl(k_p1_interp_wave<T>, (n + 255) / 256, 256, 0, s, n, p1col, blk_sys, run, xc, x);
-    else launch_pdl(k_p1_interp<T>, grid_for(n, 256, device_sms() * 16), 256, 0, s, n, p1col, blk_sys, run, xc, x);
+    const int mask = flags ? P1_MASK : 0x7fffffff;
+    if (n <= one_wave_rows<T>())
+        launch_pdl(k_p1_interp_wave<T>, (n + 255) / 256, 256, 0, s, n, p1col, mask, blk_sys, run, xc, xc2, x, x2);
+    else
+        launch_pdl(k_p1_interp<T>, grid_for(n, 256, device_sms() * 16), 256, 0, s, n, p1col, mask, blk_sys, run, xc, xc2, x,
+                   x2);
     count_launch();
 }
-template void p1_interp<float>(int, const int *, const int *, const uint8_t *, const float *, float *, cudaStream_t);
-template void p1_interp<double>(int, const int *, const int *, const uint8_t *, const double *, double *,
-                                cudaStream_t);
+template void p1_interp<float>(int, const int *, bool, const int *, const uint8_t *, const float *, const float *, float *,
+                               float *, cudaStream_t);
+template void p1_interp<double>(int, const int *, bool, const int *, const uint8_t *, const double *, const double *,
+                                double *, double *, cudaStream_t);
+
+// adds the flags to a level's columns: cf_c, the coarse level's splitting (NULL: its result is in one vector); cf, the
+// level's own (NULL: its sweeps carry all rows along)
+__global__ void k_p1_flags(int n, int *__restrict__ p1col, const int8_t *__restrict__ cf, const int8_t *__restrict__ cf_c) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        int c = p1col[i];
+        if (c < 0) continue;
+        if (cf_c && cf_c[c] == CF_C) c |= P1_SECOND;
+        if (cf && cf[i] == CF_C) c |= P1_BOTH;
+        p1col[i] = c;
+    }
+}
+
+void launch_p1_flags(int n, int *p1col, const int8_t *cf, const int8_t *cf_c, cudaStream_t s) {
+    if (n <= 0) return;
+    k_p1_flags<<<grid_for(n, 256), 256, 0, s>>>(n, p1col, cf, cf_c);
+    count_launch();
+}
 
 // ---------------------------------------------------------------------------------------
 // The bottom of the V-cycle in one launch: the restrictions of the smallest levels, the coarsest solve, and on the way

@@ -238,8 +238,12 @@ void sell_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const
 // column array (-1: no entry), which launch_p1_cols builds from P's CSR
 // blk_sys / run (batched systems, else NULL): the system of every 32-row block (-1: several) and the run flags;
 // blocks of stopped systems are skipped
+// flags: the columns carry P1_SECOND (gather from xc2 instead of xc) and P1_BOTH (write x2 as well), see sell.cu
+constexpr int P1_SECOND = 1 << 30, P1_BOTH = 1 << 29, P1_MASK = P1_BOTH - 1;
 template <class T>
-void p1_interp(int n, const int *p1col, const int *blk_sys, const uint8_t *run, const T *xc, T *x, cudaStream_t s);
+void p1_interp(int n, const int *p1col, bool flags, const int *blk_sys, const uint8_t *run, const T *xc, const T *xc2,
+               T *x, T *x2, cudaStream_t s);
+void launch_p1_flags(int n, int *p1col, const int8_t *cf, const int8_t *cf_c, cudaStream_t s);
 // the bottom of the V-cycle in one launch (sell.cu): levels of at most BOTTOM_ROWS rows, one row of a view per thread of
 // the first CTA. A level: R restricts b to the next level, P interpolates (sliced ELL, or the one-point column array
 // p1col when set), AF / AC sweep the F / C rows; the coarsest: x = Ainv b over the cluster. o_*: byte offsets in shared

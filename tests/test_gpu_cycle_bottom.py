@@ -26,6 +26,7 @@ P1 = dict(cf_mode=1, interp=1, lump_tol=0.05)
 CASES = [
     (24, dict(coarse_max=1)), (24, dict(P1, coarse_max=300)), (33, dict(coarse_max=512)), (45, dict(coarse_max=513)),
     (45, dict(P1)), (46, dict(P1)), (58, dict()), (90, dict()), (130, dict()), (150, dict(P1, coarse_max=8)),
+    (60, dict(P1, coarse_max=700)), (60, dict(P1, relax=2, coarse_max=700)),   # no bottom: split results down to the coarsest
     (181, dict(distance=2, lump_tol=0.0)), (64, dict(cf_mode=0, relax=1)), (64, dict(cf_mode=0, relax=2)),
     (100, dict(P1, relax=1)), (100, dict(P1, relax=2)),
 ]
