@@ -1229,8 +1229,8 @@ static void record_cycle(lair_handle *h, Hier &H, int l) {
 // launch-schedule autotuner for the cycle's sliced-ELL kernels (restriction, interpolation, F and C
 // sweeps): every candidate (threads per block, grid cap) is timed with CUDA events on the level's own
 // buffers (best of five), a candidate replaces the default schedule only when it is more than 5 % faster,
-// views of fewer than TUNE_MIN_ROWS rows keep the default (their few-microsecond timings alone did not carry
-// over into the captured cycle),
+// views of fewer than TUNE_MIN_ROWS rows, or that fit on the GPU in one wave and have kernels of their own, keep the
+// default (their few-microsecond timings alone did not carry over into the captured cycle),
 // and the choice is cached for the process by view shape (kind, precision, rows in quarter octaves, mean
 // row length), so later hierarchies with similar levels take it without timing. One thread owns each row
 // in these kernels, so the schedule never changes a result.

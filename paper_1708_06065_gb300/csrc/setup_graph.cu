@@ -627,16 +627,6 @@ __global__ void __launch_bounds__(32) k_rs_split(int n_all, const int2 *__restri
     }
 }
 
-// the largest number of in-block entries of S over the blocks (S and ST have the same count)
-__global__ void __launch_bounds__(32) k_rs_count(const int2 *__restrict__ blocks, Graph S, int *__restrict__ maxcnt) {
-    const int b0 = blocks[blockIdx.x].x, b1 = blocks[blockIdx.x].y;
-    int c = 0;
-    for (int i = b0 + threadIdx.x; i < b1; i += 32)
-        for (int p = S.rp[i]; p < S.rp[i + 1]; ++p) c += (S.col[p] >= b0 && S.col[p] < b1);
-    c = __reduce_add_sync(0xffffffffu, c);
-    if (threadIdx.x == 0) atomicMax(maxcnt, c);
-}
-
 // per block: the in-block entries of S (for staging), and the largest in-block row lengths of S and ST;
 // out[0..2] take the maxima over all blocks. Bound by the latency of its row reads, so a CTA of eight warps per
 // block (64^2 FD, one block of 4,096 points: 141 us with one warp, 14 us).
@@ -1297,11 +1287,6 @@ cudaError_t launch_pmis_all(int n, const Graph &S, const Graph &ST, double *w, i
 
 
 // blocks: nblocks (b0, b1) pairs on the device, every block at most Bmax points
-void launch_rs_count(const int2 *blocks, int nblocks, const Graph &S, int *maxcnt, cudaStream_t s) {
-    k_rs_count<<<nblocks, 32, 0, s>>>(blocks, S, maxcnt);
-    count_launch();
-}
-
 void launch_rs_degrees(const int2 *blocks, int nblocks, const Graph &S, const Graph &ST, int *out, cudaStream_t s) {
     k_rs_degrees<<<nblocks, RS_DEG_THREADS, 0, s>>>(blocks, S, ST, out);
     count_launch();

@@ -49,7 +49,6 @@ constexpr long long GRID_WAIT_POLLS = 1ll << 22;
 // lists: 2 n ints of scratch; ctl: 4 ints, zero
 cudaError_t launch_pmis_all(int n, const Graph &S, const Graph &ST, double *w, int8_t *cf, int8_t *newc, int *lists,
                             int *ctl, int *status, int wait_polls, cudaStream_t s);
-void launch_rs_count(const int2 *blocks, int nblocks, const Graph &S, int *maxcnt, cudaStream_t s);
 // first pass with a byte per point: blocks of at most RSB_MAX_N points with at most RSB_MAX_DEG in-block dependants each
 constexpr int RSB_MAX_N = 8192;
 constexpr int RSB_MAX_DEG = 127;   // lambda + 1 <= 2 * 127 + 1
