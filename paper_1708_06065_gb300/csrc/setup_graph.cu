@@ -3,6 +3,7 @@
 // lAIR set-up, Sec. 3.1 and Sec. 4).
 #include <cooperative_groups.h>
 
+#include "lane_quads.h"
 #include "setup_kernels.cuh"
 
 namespace lair {
@@ -707,8 +708,7 @@ __device__ __forceinline__ unsigned rsb_touch(const V &Sv, const RsbShared &q, i
     const int lane = threadIdx.x & 31;
     const unsigned rows = __ballot_sync(FULL, rb < re);
     unsigned dirty = 0;
-    for (int p = 0; rows >> p; p += 4) {   // four rows, eight lanes each
-        if (((rows >> p) & 15u) == 0) continue;
+    for (int p = next_lane_quad(rows, 0); p < 32; p = next_lane_quad(rows, p + 4)) {   // four rows, eight lanes each
         const int src = p + (lane >> 3);
         int r = __shfl_sync(FULL, rb, src) + (lane & 7);
         const int e = __shfl_sync(FULL, re, src);
