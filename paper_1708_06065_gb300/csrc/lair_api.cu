@@ -456,7 +456,8 @@ static lair_status split_points(lair_handle *h, Temps &t, int l, int n, const Gr
         // Blocks never span two batched systems.
         std::vector<int> cuts = seg_h;
         if (cuts.empty()) cuts = {0, n};
-        std::vector<int2> blocks;
+        const auto bp = std::make_shared<std::vector<int2>>();
+        std::vector<int2> &blocks = *bp;
         int Bmax = 1;
         for (size_t q = 0; q + 1 < cuts.size(); ++q) {
             const int s0 = cuts[q], s1 = cuts[q + 1];
@@ -472,12 +473,12 @@ static lair_status split_points(lair_handle *h, Temps &t, int l, int n, const Gr
         }
         int2 *bd;
         TRY(t.get(&bd, blocks.size()));
-        CU(cudaMemcpyAsync(bd, blocks.data(), sizeof(int2) * blocks.size(), cudaMemcpyHostToDevice, h->s));
+        CU(h->sources.upload(bd, bp, h->s));
         // in-block entries of S, largest in-block row lengths of S and ST: they choose the kernel and its shared memory
         int *mx, deg[3] = {0, 0, 0};
         TRY(new_counts(h, t, &mx, 3));
         launch_rs_degrees(bd, (int)blocks.size(), Scf, STcf, mx, h->s);
-        TRY(read_ints(h, mx, 3, deg));   // also keeps the host block list alive until its copy is done
+        TRY(read_ints(h, mx, 3, deg));
         if (Bmax <= RSB_MAX_N && deg[2] <= RSB_MAX_DEG) {
             CU(launch_rs_byte(bd, (int)blocks.size(), Bmax, deg[0], Scf, STcf, cf, h->status, h->s));
         } else {
@@ -924,7 +925,8 @@ struct SellPlan {
 
 static lair_status build_sells(lair_handle *h, Hier &H, std::vector<SellPlan> &plans) {
     Temps t(h);
-    std::vector<SellDesc> hd;
+    const auto hdp = std::make_shared<std::vector<SellDesc>>();
+    std::vector<SellDesc> &hd = *hdp;
     std::vector<SellPlan *> hp;
     int win = 0, lin = 0, sl = 0;
     int gp[3] = {0, 0, 0}, glin[3] = {0, 0, 0}, gsl0[2] = {0, 0}, gsl1[2] = {0, 0};
@@ -986,7 +988,7 @@ static lair_status build_sells(lair_handle *h, Hier &H, std::vector<SellPlan> &p
     TRY(t.get(&tot, 6));
     TRY(dalloc(h, &sp, (size_t)sl + 1));
     CU(cudaMemsetAsync(gsum, 0, 2 * sizeof(unsigned long long), h->s));
-    CU(cudaMemcpyAsync(dd, hd.data(), sizeof(SellDesc) * nd, cudaMemcpyHostToDevice, h->s));
+    CU(h->sources.upload(dd, hdp, h->s));
     launch_sell_prepare_multi(dd, nd, win, lin, cnt, gsum, h->s);
     for (int g = 0; g < 2; ++g) {
         if (gsl1[g] > gsl0[g]) TRY(scan(h, cnt + gsl0[g], sp + gsl0[g], gsl1[g] - gsl0[g], nullptr));
@@ -1025,8 +1027,7 @@ static lair_status build_sells(lair_handle *h, Hier &H, std::vector<SellPlan> &p
             v.dinv = d.sdinv;
         }
     }
-    CU(cudaMemcpyAsync(dd, hd.data(), sizeof(SellDesc) * nd, cudaMemcpyHostToDevice, h->s));
-    // (a copy from pageable memory is staged before cudaMemcpyAsync returns, so hd may go)
+    CU(h->sources.upload(dd, hdp, h->s));
     for (int g = 0; g < 2; ++g) launch_sell_fill_multi(dd, gp[g], gp[g + 1], glin[g], glin[g + 1], g == 0, h->s);
     H.sell_desc = dd;
     for (int g = 0; g < 3; ++g) {
@@ -1367,7 +1368,8 @@ static lair_status prepare_bottom(lair_handle *h, Hier &H) {
         if (H.lev[l].A.nr <= BOTTOM_ROWS && H.lev[l].A.nnz <= bottom_entries<T>() && nl - 1 - l <= BOTTOM_LEVELS) first = l;
     if (first < 0) return LAIR_OK;
     auto &o = H.bottom_o;
-    std::vector<BottomLevel<T>> d;
+    const auto dp = std::make_shared<std::vector<BottomLevel<T>>>();
+    std::vector<BottomLevel<T>> &d = *dp;
     for (; first <= nl - 2; ++first) {
         d.assign(nl - 1 - first, BottomLevel<T>());
         int at = 16, top = BOTTOM_SMEM;   // lists from the front, vectors from the back
@@ -1421,12 +1423,10 @@ static lair_status prepare_bottom(lair_handle *h, Hier &H) {
     if (first > nl - 2) return LAIR_OK;
     o.b0 = d[0].o_b;
     o.x0 = d[0].o_x;
-    const size_t bytes = sizeof(BottomLevel<T>) * d.size();
-    char *desc = nullptr;
-    TRY(dalloc(h, &desc, bytes));
+    BottomLevel<T> *desc = nullptr;
+    TRY(dalloc(h, &desc, d.size()));
     TRY(dalloc(h, &H.bottom_img, (size_t)BOTTOM_SMEM));
-    CU(cudaMemcpyAsync(desc, d.data(), bytes, cudaMemcpyHostToDevice, h->s));
-    // (a copy from pageable memory is staged before cudaMemcpyAsync returns, so d may go)
+    CU(h->sources.upload(desc, dp, h->s));
     H.bottom_desc = desc;
     H.bottom_first = first;
     pack_bottom<T>(h, H);
@@ -1626,6 +1626,7 @@ static lair_status build_hierarchy(lair_handle *h, Hier &H, const DCsr &A0, cons
     TRY(capture_cycle(h, H));
     tend(h, tp);
     CU(cudaStreamSynchronize(h->s));
+    h->sources.release();
     flush_timers(h);
     H.setup_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     return LAIR_OK;

@@ -17,6 +17,7 @@
 #include <string>
 #include <vector>
 
+#include "host_copies.h"
 #include "setup_kernels.cuh"
 
 namespace lair {
@@ -99,6 +100,7 @@ struct lair_handle {
     double *h_dbl = nullptr;
     void *scan_tmp = nullptr;
     size_t scan_tmp_bytes = 0;
+    lair::HostSources sources;    // host arrays that copies in flight read
     std::vector<void *> allocs;   // everything owned by the handle
     int *prod_nnz = nullptr;      // device: entry counts of the timed level-0 products (timing only)
     bool prod_fused = false;      // level 0 formed R A P in one pass
@@ -295,6 +297,7 @@ static inline void flush_timers(lair_handle *h);
 static inline lair_status sync_status(lair_handle *h) {
     CU(cudaMemcpyAsync(h->h_int, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->s));
     CU(cudaStreamSynchronize(h->s));
+    h->sources.release();
     flush_timers(h);
     int st = h->h_int[0];
     if (st != 0) {
