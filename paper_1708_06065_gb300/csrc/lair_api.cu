@@ -2142,11 +2142,15 @@ lair_status lair_precond_apply(lair_handle *h, const double *b, double *x) {
     LaunchScope ls(h);
     const int n = h->H.lev[0].A.nr;
     TRY(ensure_work(h, n, 0));
-    const bool bdev = is_device_ptr(b), xdev = is_device_ptr(x);
-    // device vectors are read and written where they are: b is read whole before x is written, so they may overlap
-    if (!bdev) CU(cudaMemcpyAsync(h->wb, b, sizeof(double) * n, cudaMemcpyHostToDevice, h->s));
-    TRY(precond(h, h->H, bdev ? b : h->wb, xdev ? x : h->wx));
-    if (!xdev) CU(cudaMemcpyAsync(x, h->wx, sizeof(double) * n, cudaMemcpyDeviceToHost, h->s));
+    const bool bin = kernels_take(b), xin = kernels_take(x);
+    // such vectors are read and written where they are: b is read whole before x is written, so they may overlap
+    if (!bin)
+        CU(cudaMemcpyAsync(h->wb, b, sizeof(double) * n,
+                           is_device_ptr(b) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->s));
+    TRY(precond(h, h->H, bin ? b : h->wb, xin ? x : h->wx));
+    if (!xin)
+        CU(cudaMemcpyAsync(x, h->wx, sizeof(double) * n,
+                           is_device_ptr(x) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->s));
     CU(cudaStreamSynchronize(h->s));
     return LAIR_OK;
 }

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "host_copies.h"
+#include "pointers.h"
 #include "setup_kernels.cuh"
 
 namespace lair {
@@ -442,16 +443,6 @@ static inline double bytes_spmv(const DCsr &M, double sv) {
 // x = P x_c with one-point P from its column array: a column per row, a gathered x_c per entry, x written
 static inline double bytes_p1(const DCsr &P, double sv) {
     return (double)P.nr * (4.0 + sv) + (double)P.nnz * sv;
-}
-
-// true for device (or managed) memory
-static inline bool is_device_ptr(const void *p) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
 // outer loops (lair_solve.cu)
