@@ -123,12 +123,14 @@ typedef struct {
                                  n must be a multiple of it; not with block_size, the Neumann restriction or
                                  batched systems. 0 or 1: off (default). */
     int autotune;             /* 1 (default): before the cycle is captured, time the launch schedules (threads
-                                 per block, grid cap) of the restriction, interpolation and sweep views that do
-                                 not fit on the GPU in one wave (more than 2,048 rows per SM with an FP32 cycle,
-                                 1,024 with FP64) and keep the fastest when it beats the default by 5 %;
-                                 choices are cached for the process by view shape, so later hierarchies of
-                                 similar levels reuse them. Results do not depend on it. 0: the fixed default
-                                 schedule everywhere. */
+                                 per block, grid cap) of the restriction, interpolation and sweep views of at
+                                 least 65,536 rows and keep the fastest when it beats the default by 5 %.
+                                 Launches of up to 2,048 rows per SM with an FP32 cycle, 1,024 with FP64 (rows
+                                 that a sweep copies included) have kernels with one schedule and are not
+                                 timed. Choices are cached for the process by what is launched, so later
+                                 hierarchies of similar levels reuse them; with timing, a timer
+                                 "tune_L<level>_<kernel>:..." names each. Results do not depend on it. 0: the
+                                 fixed default schedule everywhere. */
     int wait_polls;           /* bound on the polls of every device-side wait (the grid barriers of the
                                  cooperative PMIS kernel, levels above 8192 points); 0 (default): 4,194,304
                                  polls of the barrier word. A wait that runs out makes the call return

@@ -1152,6 +1152,19 @@ static double bytes_sweep(const Level &L, int target, double sv) {
     return nnzT * (sv + 4.0) + nT * (4.0 + 3.0 * sv) + (double)L.A.nr * sv;
 }
 
+// rows that a sweep of level l over the F (CF_F) or C points carries along (see split_levels)
+static int sweep_copies(const Level &L, int l, int target) {
+    if (target == CF_F) return L.split ? 0 : L.nc;
+    return L.split && l > 0 ? 0 : L.A.nr - L.nc;
+}
+
+template <class T>
+static void run_sweep(const Level &L, int l, int target, const T *b, const T *x, T *xo, cudaStream_t s) {
+    const int copies = sweep_copies(L, l, target);
+    if (target == CF_F) sell_sweep<T>(L.AF, L.crows, copies, b, x, xo, s);
+    else sell_sweep<T>(L.AC, L.frows, copies, b, x, xo, s);
+}
+
 template <class T>
 static void record_cycle(lair_handle *h, Hier &H, int l) {
     using B = CycleBufs<T>;
@@ -1207,7 +1220,7 @@ static void record_cycle(lair_handle *h, Hier &H, int l) {
     }
     if (tm) tend(h, t, true);
     int cur = 0;
-    const int n = L.A.nr, nc = L.nc;
+    const int n = L.A.nr;
     T *rb = B::b(L);
     if (h->o.nodal > 1) {
         // block Jacobi: x += D^{-1} b - (D^{-1} A) x
@@ -1218,8 +1231,7 @@ static void record_cycle(lair_handle *h, Hier &H, int l) {
         int tg = relax_seq[h->o.relax][k];
         if (tg < 0) break;
         t = tm ? tbegin(h, tg == CF_F ? "L0_sweep_F" : "L0_sweep_C", bytes_sweep(L, tg, sv), true) : -1;
-        if (tg == CF_F) sell_sweep<T>(L.AF, L.crows, L.split ? 0 : nc, rb, B::x(L, cur), B::x(L, 1 - cur), h->s);
-        else sell_sweep<T>(L.AC, L.frows, L.split && l > 0 ? 0 : n - nc, rb, B::x(L, cur), B::x(L, 1 - cur), h->s);
+        run_sweep<T>(L, l, tg, rb, B::x(L, cur), B::x(L, 1 - cur), h->s);
         if (tm) tend(h, t, true);
         cur ^= 1;
     }
@@ -1230,18 +1242,18 @@ static void record_cycle(lair_handle *h, Hier &H, int l) {
 // launch-schedule autotuner for the cycle's sliced-ELL kernels (restriction, interpolation, F and C
 // sweeps): every candidate (threads per block, grid cap) is timed with CUDA events on the level's own
 // buffers (best of five), a candidate replaces the default schedule only when it is more than 5 % faster,
-// views of fewer than TUNE_MIN_ROWS rows, or that fit on the GPU in one wave and have kernels of their own, keep the
-// default (their few-microsecond timings alone did not carry over into the captured cycle),
-// and the choice is cached for the process by view shape (kind, precision, rows in quarter octaves, mean
-// row length), so later hierarchies with similar levels take it without timing. One thread owns each row
-// in these kernels, so the schedule never changes a result.
+// views of fewer than TUNE_MIN_ROWS rows keep the default (their few-microsecond timings alone did not carry over into
+// the captured cycle), launches that the one-wave kernels take have one schedule, and the choice is cached for the
+// process by what is launched (kind, precision, rows in quarter octaves, mean row length, whether a sweep copies rows),
+// so later hierarchies with similar levels take it without timing. What is timed is the cycle's own launch, copies
+// included. One thread owns each row in these kernels, so the schedule never changes a result.
 // ---------------------------------------------------------------------------------------
 namespace {
 constexpr int TUNE_MIN_ROWS = 65536;
 struct TuneKey {
-    int dev, kind, fp32, rows, len;
+    int dev, kind, fp32, rows, len, copies;
     bool operator<(const TuneKey &o) const {
-        return std::tie(dev, kind, fp32, rows, len) < std::tie(o.dev, o.kind, o.fp32, o.rows, o.len);
+        return std::tie(dev, kind, fp32, rows, len, copies) < std::tie(o.dev, o.kind, o.fp32, o.rows, o.len, o.copies);
     }
 };
 std::mutex g_tune_mu;
@@ -1258,27 +1270,35 @@ static lair_status autotune_level(lair_handle *h, Hier &H, int l, cudaEvent_t e0
     Level &L = H.lev[l];
     if (L.coarsest) return LAIR_OK;
     Level &C = H.lev[l + 1];
-    const int n = L.A.nr, nc = L.nc;
+    const int n = L.A.nr;
     int dev = 0;
     CU(cudaGetDevice(&dev));
     bool cleared = false;
     const double lenA = n ? (double)L.A.nnz / n : 0.0;
-    struct Job { SellView *v; double len; };
-    const Job jobs[4] = {{&L.Rv, L.R.nr ? (double)L.R.nnz / L.R.nr : 0.0},
-                         {&L.Pv, L.P.nr ? (double)L.P.nnz / L.P.nr : 0.0}, {&L.AF, lenA}, {&L.AC, lenA}};
+    struct Job { const char *name; SellView *v; double len; int copies; };
+    const Job jobs[4] = {{"restrict", &L.Rv, L.R.nr ? (double)L.R.nnz / L.R.nr : 0.0, 0},
+                         {"interp", &L.Pv, L.P.nr ? (double)L.P.nnz / L.P.nr : 0.0, 0},
+                         {"sweep_F", &L.AF, lenA, sweep_copies(L, l, CF_F)},
+                         {"sweep_C", &L.AC, lenA, sweep_copies(L, l, CF_C)}};
     auto run = [&](int kind) {
         switch (kind) {
             case 0: sell_spmv<T>(L.Rv, B::b(L), B::b(C), h->s); break;
             case 1: sell_spmv<T>(L.Pv, B::x(C, 0), B::x(L, 0), h->s); break;
-            case 2: sell_sweep<T>(L.AF, L.crows, nc, B::b(L), B::x(L, 0), B::x(L, 1), h->s); break;
-            default: sell_sweep<T>(L.AC, L.frows, n - nc, B::b(L), B::x(L, 0), B::x(L, 1), h->s); break;
+            default: run_sweep<T>(L, l, kind == 2 ? CF_F : CF_C, B::b(L), B::x(L, 0), B::x(L, 1), h->s); break;
         }
+    };
+    // the choice as a timer "tune_L<level>_<kernel>:t<threads>b<blocks>r<rows per thread>"
+    auto report = [&](const Job &j, bool cached) {
+        if (!h->o.timing) return;
+        char nm[96];
+        snprintf(nm, sizeof nm, "tune_L%d_%s:t%db%dr%d%s", l, j.name, j.v->tb, j.v->grid, j.v->rpt, cached ? " cached" : "");
+        h->timers[timer_slot(h, nm, 0.0)].launches += 1;
     };
     for (int kind = 0; kind < 4; ++kind) {
         SellView &v = *jobs[kind].v;
-        if (v.nrows < TUNE_MIN_ROWS || v.nrows <= one_wave_rows<T>()) continue;   // one-wave views have one schedule
+        if (v.nrows < TUNE_MIN_ROWS || one_wave<T>((long long)v.nrows + jobs[kind].copies)) continue;
         const TuneKey key{dev, kind, (int)sizeof(T), (int)std::floor(4.0 * std::log2((double)v.nrows)),
-                          (int)std::lround(jobs[kind].len)};
+                          (int)std::lround(jobs[kind].len), jobs[kind].copies > 0 ? 1 : 0};
         {
             std::lock_guard<std::mutex> g(g_tune_mu);
             auto it = g_tune.find(key);
@@ -1286,6 +1306,7 @@ static lair_status autotune_level(lair_handle *h, Hier &H, int l, cudaEvent_t e0
                 v.tb = it->second.x;
                 v.grid = it->second.y;
                 v.rpt = it->second.z;
+                report(jobs[kind], true);
                 continue;
             }
         }
@@ -1326,6 +1347,7 @@ static lair_status autotune_level(lair_handle *h, Hier &H, int l, cudaEvent_t e0
         v.tb = pick.x;
         v.grid = pick.y;
         v.rpt = pick.z;
+        report(jobs[kind], false);
         std::lock_guard<std::mutex> g(g_tune_mu);
         g_tune[key] = pick;
     }
@@ -1453,9 +1475,6 @@ static void split_levels(lair_handle *h, Hier &H) {
 }
 
 static lair_status capture_cycle(lair_handle *h, Hier &H) {
-    if (h->o.precision == LAIR_MIXED) TRY(prepare_bottom<float>(h, H));
-    else TRY(prepare_bottom<double>(h, H));
-    split_levels(h, H);
     long long dummy = 0;
     long long *saved = g_launches;
     g_launches = &dummy;
@@ -1617,6 +1636,10 @@ static lair_status build_hierarchy(lair_handle *h, Hier &H, const DCsr &A0, cons
         TRY(build_sells(h, H, plans));
         tend(h, tv);
     }
+    // which levels the bottom takes and which sweeps copy rows decides what the cycle launches: before the tuner
+    if (o.precision == LAIR_MIXED) TRY(prepare_bottom<float>(h, H));
+    else TRY(prepare_bottom<double>(h, H));
+    split_levels(h, H);
     if (o.autotune) {
         tp = tbegin(h, "setup_autotune", 0.0);
         TRY(autotune_views(h, H));

@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(256) k_sell_sweep(SellView v, const int *__res
 // the first NB values and columns, the Jacobi diagonal, the row's index) into registers before it waits for that
 // kernel; then come NB gathers at once and the sum, in column order as above. x, b and xo are plain pointers: their
 // loads must stay behind the wait. More registers and fewer resident warps than the kernels above, which is why
-// larger views do not take it (one_wave_rows).
+// larger views do not take it (one_wave).
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -502,7 +502,7 @@ void p1_interp(int n, const int *p1col, bool flags, const int *blk_sys, const ui
                T *x, T *x2, cudaStream_t s) {
     if (n <= 0) return;
     const int mask = flags ? P1_MASK : 0x7fffffff;
-    if (n <= one_wave_rows<T>())
+    if (one_wave<T>(n))
         launch_pdl(k_p1_interp_wave<T>, (n + 255) / 256, 256, 0, s, n, p1col, mask, blk_sys, run, xc, xc2, x, x2);
     else
         launch_pdl(k_p1_interp<T>, grid_for(n, 256, device_sms() * 16), 256, 0, s, n, p1col, mask, blk_sys, run, xc, xc2, x,
@@ -912,7 +912,7 @@ __global__ void __launch_bounds__(WAVE_THREADS) k_sell_spmv_keep_wave(SellView v
 template <class T>
 void sell_spmv_keep(const SellView &v, const T *x, double *z, double *y, cudaStream_t s) {
     if (v.nrows <= 0) return;
-    if (v.nrows <= one_wave_rows<double>()) {
+    if (one_wave<double>(v.nrows)) {
         const int grid = (v.nrows + WAVE_THREADS - 1) / WAVE_THREADS;
         if (v.long_rows) launch_pdl(k_sell_spmv_keep_wave<T, 16>, grid, WAVE_THREADS, 0, s, v, x, z, y);
         else launch_pdl(k_sell_spmv_keep_wave<T, 8>, grid, WAVE_THREADS, 0, s, v, x, z, y);
@@ -992,7 +992,7 @@ void launch_sell_fill_multi(const SellDesc *d, int p0, int p1, int lin_beg, int 
 template <class T>
 void sell_spmv(const SellView &v, const T *x, T *y, cudaStream_t s) {
     if (v.nrows <= 0) return;
-    if (v.tb == 0 && v.nrows <= one_wave_rows<T>()) {
+    if (v.tb == 0 && one_wave<T>(v.nrows)) {
         const int grid = (v.nrows + WAVE_THREADS - 1) / WAVE_THREADS;
         if (v.long_rows) launch_pdl(k_sell_spmv_wave<T, 16>, grid, WAVE_THREADS, 0, s, v, x, y);
         else launch_pdl(k_sell_spmv_wave<T, 8>, grid, WAVE_THREADS, 0, s, v, x, y);
@@ -1012,7 +1012,7 @@ void sell_spmv(const SellView &v, const T *x, T *y, cudaStream_t s) {
 template <class T>
 void sell_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const T *x, T *xo, cudaStream_t s) {
     if (v.nrows + ncopy <= 0) return;
-    if (v.tb == 0 && v.nrows + ncopy <= one_wave_rows<T>()) {
+    if (v.tb == 0 && one_wave<T>((long long)v.nrows + ncopy)) {
         const int grid = (((v.nrows + 31) & ~31) + ncopy + WAVE_THREADS - 1) / WAVE_THREADS;
         if (v.long_rows) launch_pdl(k_sell_sweep_wave<T, 16>, grid, WAVE_THREADS, 0, s, v, copy, ncopy, b, x, xo);
         else launch_pdl(k_sell_sweep_wave<T, 8>, grid, WAVE_THREADS, 0, s, v, copy, ncopy, b, x, xo);

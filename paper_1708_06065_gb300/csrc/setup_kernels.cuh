@@ -226,8 +226,8 @@ struct SellDesc {
 void launch_sell_prepare_multi(const SellDesc *d, int nd, int nwin, int nlin, int *cnt, unsigned long long *gsum,
                                cudaStream_t s);
 void launch_sell_fill_multi(const SellDesc *d, int p0, int p1, int lin_beg, int lin_end, bool fp32, cudaStream_t s);
-// the largest view that the one-wave kernels take
-template <class T> long long one_wave_rows() { return (long long)device_sms() * (WAVE_BYTES_PER_SM / (int)sizeof(T)); }
+// whether the one-wave kernels take a launch over so many rows (those of the view and those copied)
+template <class T> bool one_wave(long long rows) { return rows <= (long long)device_sms() * (WAVE_BYTES_PER_SM / (int)sizeof(T)); }
 template <class T> void sell_spmv(const SellView &v, const T *x, T *y, cudaStream_t s);
 // y = A x for an FP64 view of all rows of A and an x in T, and z = x in FP64
 template <class T> void sell_spmv_keep(const SellView &v, const T *x, double *z, double *y, cudaStream_t s);
