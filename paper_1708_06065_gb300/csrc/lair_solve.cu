@@ -132,8 +132,8 @@ static lair_status solve_dev(lair_handle *h, Hier &H, const double *b, double *x
                 TRY(run_cycle(h, H));   // of v_j
                 ++it;
                 int ts = tbegin(h, "outer_spmv", bytes_spmv(A, 8.0));
-                if (mixed) sell_spmv_keep<float>(L0.A64, L0.x32[L0.xfinal], zj, w, h->s);
-                else sell_spmv_keep<double>(L0.A64, L0.x64[L0.xfinal], zj, w, h->s);
+                if (mixed) sell_spmv_keep<float>(L0.A64, A.nnz, L0.x32[L0.xfinal], zj, w, h->s);
+                else sell_spmv_keep<double>(L0.A64, A.nnz, L0.x64[L0.xfinal], zj, w, h->s);
                 tend(h, ts);
                 int to = tbegin(h, "outer_cgs2", 8.0 * n * (3.0 * (j + 2) + 4.0));
                 cgs2(n, j + 1, V, n, w, h->part, hbuf, hbuf + 32, hsum, nrm, inv, h->s);
@@ -423,8 +423,8 @@ lair_status solve_batched_fgmres(lair_handle *h, Hier &H, const double *b, doubl
             double *zj = Z + (size_t)j * n, *w = V + (size_t)(j + 1) * n;
             TRY(run_cycle(h, H));   // of v_j
             int ts = tbegin(h, "outer_spmv", bytes_spmv(A, 8.0));
-            if (mixed) sell_spmv_keep<float>(L0.A64, L0.x32[L0.xfinal], zj, w, h->s);
-            else sell_spmv_keep<double>(L0.A64, L0.x64[L0.xfinal], zj, w, h->s);
+            if (mixed) sell_spmv_keep<float>(L0.A64, A.nnz, L0.x32[L0.xfinal], zj, w, h->s);
+            else sell_spmv_keep<double>(L0.A64, A.nnz, L0.x64[L0.xfinal], zj, w, h->s);
             tend(h, ts);
             // CGS2 in three streaming passes over V: dots; update and dots; update and norm
             seg_cgs_pass(sta, 1, j + 1, V, n, HS, nullptr, w, hbuf, hsum, h->s);

@@ -258,13 +258,12 @@ __global__ void __launch_bounds__(256) k_sell_spmv(SellView v, const T *__restri
         int lmax = 0;
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
-            bool on = s0 + k < nsl, zero = false;
+            bool on = s0 + k < nsl;
             if (on && v.run) {
                 const int q = v.slice_sys[s0 + k];
                 on = q < 0 || v.run[q];
-                zero = !on && v.zero_stopped;   // no entries: the row's sum stays 0 and is written
             }
-            r[k] = on || zero ? (s0 + k) * 32 + lane : v.nrows;
+            r[k] = on ? (s0 + k) * 32 + lane : v.nrows;
             base[k] = 0;
             len[k] = 0;
             if (on) {
@@ -356,45 +355,48 @@ __global__ void __launch_bounds__(256) k_sell_sweep(SellView v, const int *__res
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// An entry stays in registers from here on: left alone, the compiler may move its loads past the wait into the branch
+// that uses them (FP64 sweeps with 32 instead of 88 registers; 301^2 FD, solve 3.14 -> 3.20 ms).
+__device__ __forceinline__ void hold(int &c, float &w) { asm volatile("" : "+r"(c), "+f"(w)); }
+__device__ __forceinline__ void hold(int &c, double &w) { asm volatile("" : "+r"(c), "+d"(w)); }
+
 template <class T, int NB>
 struct RowHead {
     int base = 0, len = 0, i = -1;
     int c[NB];
     T w[NB];
-    // row slot u of the view (u < 32 * slices); a slice of a stopped system has no row, or a row without entries when
-    // its rows are to be written as 0
+    // row slot u of the view (u < 32 * slices); a slice of a stopped system has no row
     __device__ __forceinline__ void load(const SellView &v, int u, int nrows) {
         const int sl = u >> 5, lane = u & 31;
-        bool on = true, zero = false;
+        bool on = true;
         if (v.run) {
             const int q = v.slice_sys[sl];
             on = q < 0 || v.run[q];
-            zero = !on && v.zero_stopped;
         }
         if (on) {
             const int a = __ldg(v.slice_ptr + sl);
             base = a + lane;
             len = (__ldg(v.slice_ptr + sl + 1) - a) >> 5;
         }
-        if ((on || zero) && u < nrows) i = __ldg(v.row + u);
+        if (on && u < nrows) i = __ldg(v.row + u);
         const T *val = static_cast<const T *>(v.val);
 #pragma unroll
         for (int k = 0; k < NB; ++k) {
             c[k] = k < len ? __ldg(v.col + base + 32 * k) : 0;
             w[k] = k < len ? __ldg(val + base + 32 * k) : T(0);
         }
+#pragma unroll
+        for (int k = 0; k < NB; ++k) hold(c[k], w[k]);
     }
-    // (x in X: T, or FP32 widened to T)
-    template <class X>
-    __device__ __forceinline__ T sum(const SellView &v, const X *x) const {
+    __device__ __forceinline__ T sum(const SellView &v, const T *x) const {
         T acc = T(0);
         {
-            X xv[NB];
+            T xv[NB];
 #pragma unroll
-            for (int k = 0; k < NB; ++k) xv[k] = k < len ? x[c[k]] : X(0);
+            for (int k = 0; k < NB; ++k) xv[k] = k < len ? x[c[k]] : T(0);
 #pragma unroll
             for (int k = 0; k < NB; ++k)
-                if (k < len) acc = fma(w[k], (T)xv[k], acc);
+                if (k < len) acc = fma(w[k], xv[k], acc);
         }
         const T *val = static_cast<const T *>(v.val);
         for (int j = NB; j < len; j += NB) {
@@ -407,7 +409,7 @@ struct RowHead {
             }
 #pragma unroll
             for (int k = 0; k < NB; ++k)
-                if (j + k < len) acc = fma(ww[k], (T)x[cc[k]], acc);
+                if (j + k < len) acc = fma(ww[k], x[cc[k]], acc);
         }
         return acc;
     }
@@ -868,9 +870,9 @@ void launch_p1_cols(int n, const int *rp, const int *col, int *p1col, cudaStream
     count_launch();
 }
 
-// The outer iteration's product y = A z with z = the cycle's result x (FP32, widened exactly, or FP64), which the
-// kernel also writes out: one launch instead of a conversion and a product, and in mixed precision the gathers read
-// half the bytes. The arithmetic of k_sell_spmv<double>.
+// The outer iteration's product y = A z with z = the cycle's result x (FP32, widened exactly, or FP64), which is also
+// written out: in one kernel, whose gathers read half the bytes in mixed precision, or as a conversion and
+// k_sell_spmv<double>, whose arithmetic the kernel has.
 template <class T>
 __global__ void __launch_bounds__(256) k_sell_spmv_keep(SellView v, const T *x, double *z, double *y) {
     pdl_enter();
@@ -885,7 +887,7 @@ __global__ void __launch_bounds__(256) k_sell_spmv_keep(SellView v, const T *x, 
             on = sy < 0 || v.run[sy];
         }
         const int a = __ldg(sptr + sl), base = a + (q & 31);
-        const int len = on ? (__ldg(sptr + sl + 1) - a) >> 5 : 0;   // a stopped system: y = 0
+        const int len = on ? (__ldg(sptr + sl + 1) - a) >> 5 : 0;   // a stopped system: y = 0, which nothing reads
         const int i = __ldg(v.row + q);
         double acc = 0.0;
 #pragma unroll 4
@@ -895,34 +897,32 @@ __global__ void __launch_bounds__(256) k_sell_spmv_keep(SellView v, const T *x, 
     }
 }
 
-template <class T, int NB>
-__global__ void __launch_bounds__(WAVE_THREADS) k_sell_spmv_keep_wave(SellView v, const T *x, double *z, double *y) {
-    pdl_launch_next();
-    const int u = blockIdx.x * WAVE_THREADS + threadIdx.x;
-    RowHead<double, NB> h;
-    if (u < ((v.nrows + 31) & ~31)) h.load(v, u, v.nrows);
-    pdl_wait_previous();
-    const double acc = h.sum(v, x);
-    if (h.i >= 0) {
-        y[h.i] = acc;
-        z[h.i] = (double)x[h.i];
-    }
-}
+// Both ways give the same bits. Which one: the fused kernel converts x once per entry, on FP64 units that take as long
+// for a conversion as for an fma, the pair once per row; the pair costs a launch and reads x again. In mixed precision
+// they cross at about KEEP_ENTRIES_PER_SM entries (us, fused / pair): 300^2 8.0 / 10.6, 512^2 11.9 / 12.5, 700^2 17.2 /
+// 17.2, 900^2 23.7 / 22.3; 42^3 8.6 / 10.8, 53^3 11.1 / 12.3, 64^3 13.8 / 13.2, 101^3 36 / 30, 150^3 107 / 74; DG-P2 64^2
+// 9.6 / 11.7, 90^2 11.6 / 12.7, 110^2 13.7 / 13.4, 150^2 17.9 / 16.0, 256^2 40 / 31. Batches keep the fused kernel, which
+// does not work on systems that have stopped (512 systems, mean of all iterations: 123.5 / 125.3). A form with one row
+// per thread and the matrix read ahead, as in the cycle, was slower: 53^3 16.8, FP64 11.9 against 9.4.
+constexpr int KEEP_ENTRIES_PER_SM = 10240;
 
 template <class T>
-void sell_spmv_keep(const SellView &v, const T *x, double *z, double *y, cudaStream_t s) {
+void sell_spmv_keep(const SellView &v, long long nnz, const T *x, double *z, double *y, cudaStream_t s) {
     if (v.nrows <= 0) return;
-    if (one_wave<double>(v.nrows)) {
-        const int grid = (v.nrows + WAVE_THREADS - 1) / WAVE_THREADS;
-        if (v.long_rows) launch_pdl(k_sell_spmv_keep_wave<T, 16>, grid, WAVE_THREADS, 0, s, v, x, z, y);
-        else launch_pdl(k_sell_spmv_keep_wave<T, 8>, grid, WAVE_THREADS, 0, s, v, x, z, y);
-    } else {
-        launch_pdl(k_sell_spmv_keep<T>, grid_for(v.nrows, 256, device_sms() * 16), 256, 0, s, v, x, z, y);
+    const int grid = grid_for(v.nrows, 256, device_sms() * 16);
+    if constexpr (sizeof(T) == 4) {
+        if (!v.run && nnz > (long long)KEEP_ENTRIES_PER_SM * device_sms()) {
+            f2d(v.nrows, x, z, s);
+            launch_pdl(k_sell_spmv<double, 1>, grid, 256, 0, s, v, (const double *)z, y);
+            count_launch();
+            return;
+        }
     }
+    launch_pdl(k_sell_spmv_keep<T>, grid, 256, 0, s, v, x, z, y);
     count_launch();
 }
-template void sell_spmv_keep<float>(const SellView &, const float *, double *, double *, cudaStream_t);
-template void sell_spmv_keep<double>(const SellView &, const double *, double *, double *, cudaStream_t);
+template void sell_spmv_keep<float>(const SellView &, long long, const float *, double *, double *, cudaStream_t);
+template void sell_spmv_keep<double>(const SellView &, long long, const double *, double *, double *, cudaStream_t);
 
 // r = b - A x over all rows of an FP64 view of A (r and its FP32 copy each optional), and the block partial
 // of |r|^2 in part[blockIdx.x] (gridDim.x = RED_PARTS blocks, summed by finish_residual)

@@ -20,7 +20,6 @@ struct SellView {
     // slices of a stopped system are skipped (their outputs keep older values). NULL: every slice runs.
     const int *slice_sys = nullptr;
     const uint8_t *run = nullptr;
-    bool zero_stopped = false;  // products: write 0 to the rows of a stopped system's slices instead of skipping them
 };
 
 // One-wave kernels (sell.cu): views of at most WAVE_BYTES_PER_SM / sizeof(T) rows per SM (2,048 in FP32, a full SM of
@@ -229,8 +228,8 @@ void launch_sell_fill_multi(const SellDesc *d, int p0, int p1, int lin_beg, int 
 // whether the one-wave kernels take a launch over so many rows (those of the view and those copied)
 template <class T> bool one_wave(long long rows) { return rows <= (long long)device_sms() * (WAVE_BYTES_PER_SM / (int)sizeof(T)); }
 template <class T> void sell_spmv(const SellView &v, const T *x, T *y, cudaStream_t s);
-// y = A x for an FP64 view of all rows of A and an x in T, and z = x in FP64
-template <class T> void sell_spmv_keep(const SellView &v, const T *x, double *z, double *y, cudaStream_t s);
+// y = A x for an FP64 view of all rows of A (nnz entries) and an x in T, and z = x in FP64
+template <class T> void sell_spmv_keep(const SellView &v, long long nnz, const T *x, double *z, double *y, cudaStream_t s);
 template <class T>
 void sell_sweep(const SellView &v, const int *copy, int ncopy, const T *b, const T *x, T *xo, cudaStream_t s);
 // x = P x_c for a P with at most one entry per row, every entry 1 (one-point interpolation), from its dense
