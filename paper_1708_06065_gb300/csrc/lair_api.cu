@@ -474,12 +474,12 @@ static lair_status split_points(lair_handle *h, Temps &t, int l, int n, const Gr
         int2 *bd;
         TRY(t.get(&bd, blocks.size()));
         CU(h->sources.upload(bd, bp, h->s));
-        // in-block entries of S, largest in-block row lengths of S and ST: they choose the kernel and its shared memory
-        int *mx, deg[3] = {0, 0, 0};
-        TRY(new_counts(h, t, &mx, 3));
+        // in-block entries of S and the largest in-block row length of ST: they choose the kernel and its shared memory
+        int *mx, deg[2] = {0, 0};
+        TRY(new_counts(h, t, &mx, 2));
         launch_rs_degrees(bd, (int)blocks.size(), Scf, STcf, mx, h->s);
-        TRY(read_ints(h, mx, 3, deg));
-        if (Bmax <= RSB_MAX_N && deg[2] <= RSB_MAX_DEG) {
+        TRY(read_ints(h, mx, 2, deg));
+        if (Bmax <= RSB_MAX_N && deg[1] <= RSB_MAX_DEG) {
             CU(launch_rs_byte(bd, (int)blocks.size(), Bmax, deg[0], Scf, STcf, cf, h->status, h->s));
         } else {
             CU(launch_rs(n, bd, (int)blocks.size(), Bmax, deg[0], Scf, STcf, cf, h->status, h->s));

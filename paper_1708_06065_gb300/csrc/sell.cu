@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(WAVE_THREADS) k_sell_sweep_wave(SellView v, co
 // that the sliced-ELL product gives (a -0 becomes +0). One column per row from the dense column array, one
 // gather, one write: coalesced everywhere but the gather.
 //
-// Two flags above the column (P1_MASK) spare the sweeps their copies of the rows they do not touch (split_p1_cols):
+// Two flags above the column (P1_MASK) spare the sweeps their copies of the rows they do not touch (split_levels):
 // P1_SECOND: the coarse point is a C point of a level whose result lies in two vectors, F points in the first and C
 // points in the second; P1_BOTH: the row is a C point, written to x and x2, so that the F sweeps can go from one to the
 // other without carrying the C points along.

@@ -628,8 +628,8 @@ __global__ void __launch_bounds__(32) k_rs_split(int n_all, const int2 *__restri
     }
 }
 
-// per block: the in-block entries of S (for staging), and the largest in-block row lengths of S and ST;
-// out[0..2] take the maxima over all blocks. Bound by the latency of its row reads, so a CTA of eight warps per
+// per block: the in-block entries of S (for staging), and the largest in-block row length of ST; out[0..1] take the
+// maxima over all blocks. Bound by the latency of its row reads, so a CTA of eight warps per
 // block (64^2 FD, one block of 4,096 points: 141 us with one warp, 14 us).
 constexpr int RS_DEG_THREADS = 256;
 
@@ -639,22 +639,19 @@ __global__ void __launch_bounds__(RS_DEG_THREADS) k_rs_degrees(const int2 *__res
     const int b0 = blocks[blockIdx.x].x, b1 = blocks[blockIdx.x].y;
     if (threadIdx.x == 0) total = 0;
     __syncthreads();
-    int c = 0, ms = 0, mt = 0;
+    int c = 0, mt = 0;
     for (int i = b0 + threadIdx.x; i < b1; i += RS_DEG_THREADS) {
-        int ds = 0, dt = 0;
+        int ds = 0, dt = 0;   // of S and ST
         for (int p = S.rp[i]; p < S.rp[i + 1]; ++p) ds += (S.col[p] >= b0 && S.col[p] < b1);
         for (int p = ST.rp[i]; p < ST.rp[i + 1]; ++p) dt += (ST.col[p] >= b0 && ST.col[p] < b1);
         c += ds;
-        ms = max(ms, ds);
         mt = max(mt, dt);
     }
     c = __reduce_add_sync(0xffffffffu, c);
-    ms = __reduce_max_sync(0xffffffffu, ms);
     mt = __reduce_max_sync(0xffffffffu, mt);
     if ((threadIdx.x & 31) == 0) {
         atomicAdd(&total, c);
-        atomicMax(&out[1], ms);
-        atomicMax(&out[2], mt);
+        atomicMax(&out[1], mt);
     }
     __syncthreads();
     if (threadIdx.x == 0) atomicMax(&out[0], total);
