@@ -10,12 +10,11 @@
 
 namespace lair {
 
-// The first lane of the first group at or after lane p (a multiple of 4, at most 32) of which any lane is in `lanes`,
-// or 32. The mask is shifted by less than its width only: by 32, which p reaches when one of lanes 28 to 31 is in the
-// mask, a shift is undefined (the GPU's gives 0, x86's leaves the mask as it is).
-LAIR_HD constexpr int next_lane_quad(unsigned lanes, int p) {
-    while (p < 32 && ((lanes >> p) & 15u) == 0) p += 4;
-    return p;
-}
+// A walk over the groups that have a lane in the mask:
+//   for (int p = 0; lanes_from(lanes, p); p += 4) if (lane_quad(lanes, p)) ...
+// The mask is shifted by less than its width only: by 32, which p reaches when one of lanes 28 to 31 is in the mask, a
+// shift is undefined (the GPU's gives 0, x86's leaves the mask as it is).
+LAIR_HD constexpr bool lanes_from(unsigned lanes, int p) { return p < 32 && lanes >> p != 0; }
+LAIR_HD constexpr bool lane_quad(unsigned lanes, int p) { return ((lanes >> p) & 15u) != 0; }   // p < 32
 
 }  // namespace lair

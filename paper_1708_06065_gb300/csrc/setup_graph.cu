@@ -705,7 +705,8 @@ __device__ __forceinline__ unsigned rsb_touch(const V &Sv, const RsbShared &q, i
     const int lane = threadIdx.x & 31;
     const unsigned rows = __ballot_sync(FULL, rb < re);
     unsigned dirty = 0;
-    for (int p = next_lane_quad(rows, 0); p < 32; p = next_lane_quad(rows, p + 4)) {   // four rows, eight lanes each
+    for (int p = 0; lanes_from(rows, p); p += 4) {   // four rows, eight lanes each
+        if (!lane_quad(rows, p)) continue;
         const int src = p + (lane >> 3);
         int r = __shfl_sync(FULL, rb, src) + (lane & 7);
         const int e = __shfl_sync(FULL, re, src);

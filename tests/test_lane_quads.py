@@ -12,8 +12,9 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 PROGRAM = r"""
 #include "lane_quads.h"
 // constant evaluation refuses undefined operations
-static_assert(lair::next_lane_quad(0xffffffffu, 32) == 32, "end");
-static_assert(lair::next_lane_quad(0x80000000u, 0) == 28 && lair::next_lane_quad(0u, 0) == 32, "last group, none");
+static_assert(!lair::lanes_from(0xffffffffu, 32), "end");
+static_assert(lair::lanes_from(0x80000000u, 28) && lair::lane_quad(0x80000000u, 28), "last group");
+static_assert(!lair::lanes_from(0u, 0) && !lair::lanes_from(0xfu, 4) && !lair::lane_quad(0xfffffff0u, 0), "none");
 int main() {
     for (unsigned groups = 0; groups < 256; ++groups)
         for (int lane = 0; lane < 4; ++lane) {   // the lane that stands for its group
@@ -21,8 +22,9 @@ int main() {
             for (int g = 0; g < 8; ++g)
                 if (groups >> g & 1) lanes |= 1u << (4 * g + lane);
             int last = -4, steps = 0;
-            for (int p = lair::next_lane_quad(lanes, 0); p < 32; p = lair::next_lane_quad(lanes, p + 4)) {
+            for (int p = 0; lair::lanes_from(lanes, p); p += 4) {
                 if (p % 4 || p <= last || ++steps > 8) return 1;
+                if (!lair::lane_quad(lanes, p)) continue;
                 last = p;
                 seen |= 1u << (p / 4);
             }
