@@ -1204,7 +1204,7 @@ static void record_cycle(lair_handle *h, Hier &H, int l) {
     if (tm) tend(h, t, true);
     record_cycle<T>(h, H, l + 1);
     const bool p1 = h->o.interp == LAIR_P_ONEPOINT && L.p1col;
-    t = tm ? tbegin(h, "L0_interp", p1 ? bytes_p1(L.P, sv) : bytes_spmv(L.P, sv), true) : -1;
+    t = tm ? tbegin(h, "L0_interp", p1 ? bytes_p1(L.P, sv, L.split ? L.nc : 0) : bytes_spmv(L.P, sv), true) : -1;
     if (p1) {
         // at most one entry per row of P, every entry 1 (one-point, or the identity blocks of the nodal one-point
         // P): the direct kernel on the dense column array, rows in their own order

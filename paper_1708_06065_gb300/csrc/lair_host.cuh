@@ -440,9 +440,10 @@ static inline lair_status new_counts(lair_handle *h, Temps &t, int **p, int n) {
 static inline double bytes_spmv(const DCsr &M, double sv) {
     return (double)M.nnz * (sv + 4.0) + (double)M.nr * (4.0 + sv) + (double)M.nc * sv;
 }
-// x = P x_c with one-point P from its column array: a column per row, a gathered x_c per entry, x written
-static inline double bytes_p1(const DCsr &P, double sv) {
-    return (double)P.nr * (4.0 + sv) + (double)P.nnz * sv;
+// x = P x_c with one-point P from its column array: a column per row, a gathered x_c per entry, x written, and `both` of
+// its rows once more into the second x buffer
+static inline double bytes_p1(const DCsr &P, double sv, int both) {
+    return (double)P.nr * (4.0 + sv) + ((double)P.nnz + both) * sv;
 }
 
 // outer loops (lair_solve.cu)
