@@ -345,13 +345,13 @@ __global__ void __launch_bounds__(256) k_sell_sweep(SellView v, const int *__res
     }
 }
 
-// The same product and sweep for views whose rows fit on the GPU in one wave. There a launch is bound by its chain of
+// The same product and sweep for launches of about one wave (one_wave). Those are bound by their chain of
 // dependent loads -- slice offset, columns, gathered x, then row and b -- and by the launch itself, not by bandwidth.
 // So a thread has one row and brings everything that does not depend on the previous kernel of the cycle (offsets,
 // the first NB values and columns, the Jacobi diagonal, the row's index) into registers before it waits for that
 // kernel; then come NB gathers at once and the sum, in column order as above. x, b and xo are plain pointers: their
 // loads must stay behind the wait. More registers and fewer resident warps than the kernels above, which is why
-// larger views do not take it (one_wave).
+// larger views do not take it.
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(256) k_p1_interp(int n, const int *__restrict_
     }
 }
 
-// the same in one wave, a row per thread: the column is read before the previous kernel has finished
+// the same for about one wave, a row per thread: the column is read before the previous kernel has finished
 template <class T>
 __global__ void __launch_bounds__(256) k_p1_interp_wave(int n, const int *p1col, int mask, const int *blk_sys,
                                                         const uint8_t *run, const T *xc, const T *xc2, T *x, T *x2) {

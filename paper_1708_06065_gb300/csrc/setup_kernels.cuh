@@ -14,7 +14,7 @@ struct SellView {
     int *row = nullptr;         // view row -> matrix row
     void *dinv = nullptr;       // Jacobi diagonal per view row (sweep views), same type as val
     int tb = 0, grid = 0;       // launch schedule picked by the autotuner (0: 256 threads, grid capped at 16 blocks per SM)
-    bool long_rows = false;     // more than WAVE_SHORT entries a row on average (the one-wave kernels' variants)
+    bool long_rows = false;     // more than WAVE_SHORT entries a row on average (the variants of the one-wave kernels)
     int rpt = 1;                // rows per thread (1 or 2: rows of two consecutive slices, same lane)
     // batched systems: the system of every slice (-1: rows of several systems) and the per-system run flags;
     // slices of a stopped system are skipped (their outputs keep older values). NULL: every slice runs.
@@ -22,11 +22,14 @@ struct SellView {
     const uint8_t *run = nullptr;
 };
 
-// One-wave kernels (sell.cu): views of at most WAVE_BYTES_PER_SM / sizeof(T) rows per SM (2,048 in FP32, a full SM of
-// threads; 1,024 in FP64, whose registers allow half of that); rows of more than WAVE_SHORT entries on average read 16
-// entries ahead instead of 8. V-cycle with 0 / 512 / 1,024 / 2,048 / 4,096 FP32 rows per SM: 512^2 FD 152 / 134 / 128 /
-// 121 / 120 us, 128^3 314 / 304 / 292 / 281 / 279 us; FP64 0 / 512 / 1,024 / 2,048: 101^3 299 / 273 / 259 / 253 us,
-// 24 systems 253 / 222 / 217 / 223 us.
+// One-wave kernels (sell.cu): launches over at most WAVE_BYTES_PER_SM / sizeof(T) rows per SM, 2,048 in FP32 and 1,024 in
+// FP64. The limit is a measured one: by their registers (40 to 88 a thread) an SM holds 1,536 to 640 of their threads,
+// and a launch near the limit takes up to two waves. V-cycle with 0 / 512 / 1,024 / 2,048 / 4,096 FP32 rows per SM: 512^2
+// FD 152 / 134 / 128 / 121 / 120 us, 128^3 314 / 304 / 292 / 281 / 279 us; FP64 0 / 512 / 1,024 / 2,048: 101^3 299 / 273 /
+// 259 / 253 us, 24 systems 253 / 222 / 217 / 223 us.
+// Rows of more than WAVE_SHORT entries on average read 16 entries ahead instead of 8. V-cycle with 16 for all rows / this
+// / 8 for all: 256^2 FD 90 / 85 / 84 us, 512^2 105 / 100 / 100, 300^2 FP64 124 / 110 / 109, 128^3 248 / 255 / 257, DG-P2
+// 128^2 102 / 106 / 108, 300^2 lAIP FP64 184 / 176 / 181.
 constexpr int WAVE_SHORT = 6;
 constexpr int WAVE_BYTES_PER_SM = 8192;
 
@@ -272,8 +275,9 @@ constexpr int BOTTOM_THREADS = 1024;
 constexpr int BOTTOM_ROWS = BOTTOM_THREADS;
 // Entries of A that a level of the bottom may have: with more, one SM's shared memory (FP32) or its two FP64 lanes cost
 // more than the kernel boundaries that the bottom saves. V-cycle with limits of 1,000 / 4,096 / 8,192 / 20,000 entries
-// in FP64: 301^2 FD lAIP 174 / 174 / 165 / 170 us, 64^2 87 / 85 / 81 / 81 us; in FP32 2,000 / 5,000 / 12,288 / 20,000:
-// 512^2 FD one-point 101 / 96 / 98 / 97 us; without a bottom 177, 88 and 107 us.
+// in FP64: 301^2 FD lAIP 174 / 174 / 165 / 170 us, 64^2 87 / 85 / 81 / 81 us; in FP32 5,000 / 8,192 / 12,288: 64^2 FD lAIP
+// 78 / 72 / 69 us, 128^2 94 / 87 / 86, 301^2 125 / 116 / 114, with one-point P the same to 2 us (512^2 100 / 100 / 99);
+// 20,000 with one-point P: 97 against 98 us at 512^2.
 template <class T> constexpr int bottom_entries() { return sizeof(T) == 4 ? 12288 : 8192; }
 constexpr int BOTTOM_LEVELS = 25;                // more levels than this are not taken into the bottom
 // Half of an SM's on-chip memory: with 224 KB the SMs that ran the bottom were left without an L1 for the streaming
